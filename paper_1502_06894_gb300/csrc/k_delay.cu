@@ -21,10 +21,15 @@
 
 namespace corr {
 
-__global__ void k_delay_blocks(DelayParams p) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+constexpr int kDelayThreads = 128;
+
+__global__ void __launch_bounds__(kDelayThreads) k_delay_blocks(DelayParams p) {
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
   const int s = blockIdx.y;
-  if (i >= p.nb) return;
+  // threads beyond the last block repeat it (they write nothing), so that
+  // whole warps reach the reductions below
+  const bool mine = i0 < p.nb;
+  const int i = mine ? i0 : p.nb - 1;
   const int64_t b = p.b0 + i;
   const int N = p.N;
   const double tc = __ddiv_rn((double)(b * (int64_t)N + N / 2), p.fs);
@@ -53,16 +58,18 @@ __global__ void k_delay_blocks(DelayParams p) {
     for (int64_t f = qa / v.payload; f <= qb / v.payload && ok; ++f) ok = f < v.nframes && v.frame_ok[f] != 0;
   }
   const size_t o = (size_t)s * p.ld + i;
-  p.start[o] = start;
-  p.valid[o] = ok ? 1 : 0;
-  p.delta[o] = (float)__ddiv_rn(__dmul_rn(eps, p.fs), (double)N);
+  if (mine) {
+    p.start[o] = start;
+    p.valid[o] = ok ? 1 : 0;
+    p.delta[o] = (float)__ddiv_rn(__dmul_rn(eps, p.fs), (double)N);
+  }
   // pre-F rotation: the delay rate at t_c (derivative of the same segment)
   double rate = 0.0;
   if (p.dphi) {
 #pragma unroll
     for (int q = 5; q >= 1; --q) rate = __fma_rn(rate, u, (double)q * c[q]);
   }
-  for (int sb = 0; sb < p.nsub; ++sb) {
+  for (int sb = 0; mine && sb < p.nsub; ++sb) {
     double ph = __dmul_rn(p.nu0[sb], tau);
     ph = __dsub_rn(ph, floor(ph));
     const size_t os = ((size_t)s * p.nsub + sb) * p.ld + i;
@@ -86,16 +93,41 @@ __global__ void k_delay_blocks(DelayParams p) {
       p.phi[os] = (float)ph;
     }
   }
-  if (p.eps_out) p.eps_out[o] = eps;
-  if (p.tau_out) p.tau_out[o] = tau;
+  if (mine && p.eps_out) p.eps_out[o] = eps;
+  if (mine && p.tau_out) p.tau_out[o] = tau;
   if (p.max_end) {
     // [0]: max window end, [1]: min window start (both relative to the
     // station's first sample, offset by 2^62 so they order as unsigned);
-    // [2]: number of valid blocks.
+    // [2]: number of valid blocks.  Reduced over the CTA first: one atomic of
+    // every thread on the station's three words serialised the kernel
+    // (62500 blocks x 2 stations: 169 us, 17.7 us now).
     const unsigned long long off = 1ull << 62;
-    atomicMax(&p.max_end[3 * s + 0], (unsigned long long)(rel + N) + off);
-    atomicMin(&p.max_end[3 * s + 1], (unsigned long long)rel + off);
-    if (ok) atomicAdd(&p.max_end[3 * s + 2], 1ull);
+    unsigned long long hi = (unsigned long long)(rel + N) + off, lo = (unsigned long long)rel + off;
+    const int count = __popc(__ballot_sync(0xffffffffu, mine && ok));
+    for (int q = 16; q > 0; q >>= 1) {
+      const unsigned long long h2 = __shfl_down_sync(0xffffffffu, hi, q), l2 = __shfl_down_sync(0xffffffffu, lo, q);
+      hi = h2 > hi ? h2 : hi;
+      lo = l2 < lo ? l2 : lo;
+    }
+    __shared__ unsigned long long s_hi[kDelayThreads / 32], s_lo[kDelayThreads / 32];
+    __shared__ int s_count[kDelayThreads / 32];
+    if ((threadIdx.x & 31) == 0) {
+      s_hi[threadIdx.x >> 5] = hi;
+      s_lo[threadIdx.x >> 5] = lo;
+      s_count[threadIdx.x >> 5] = count;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int total = s_count[0];
+      for (int w = 1; w < kDelayThreads / 32; ++w) {
+        hi = s_hi[w] > hi ? s_hi[w] : hi;
+        lo = s_lo[w] < lo ? s_lo[w] : lo;
+        total += s_count[w];
+      }
+      atomicMax(&p.max_end[3 * s + 0], hi);
+      atomicMin(&p.max_end[3 * s + 1], lo);
+      if (total) atomicAdd(&p.max_end[3 * s + 2], (unsigned long long)total);
+    }
   }
 }
 
@@ -127,8 +159,8 @@ cudaError_t launch_deframe(const uint8_t* raw, int payload, int64_t f0, int64_t 
 
 cudaError_t launch_delay_blocks(const DelayParams& p, cudaStream_t s) {
   if (p.nb <= 0) return cudaSuccess;
-  dim3 grid((p.nb + 127) / 128, p.S);
-  k_delay_blocks<<<grid, 128, 0, s>>>(p);
+  dim3 grid((p.nb + kDelayThreads - 1) / kDelayThreads, p.S);
+  k_delay_blocks<<<grid, kDelayThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 

@@ -10,7 +10,11 @@
 
 namespace corr {
 
-__global__ void k_weights(FinParams p) {
+// One CTA per baseline.  Bound by the latency of its loads, which take 16
+// blocks each where the rows of `valid` start at multiples of 16 bytes (a
+// handle pads them; the static scratch has no room to): 62500 blocks took 120
+// us with byte loads, 11.2 us now.
+__global__ void __launch_bounds__(256) k_weights(FinParams p) {
   const int bl = blockIdx.x;
   // decode baseline index -> (a, b)
   int a = 0, q = bl;
@@ -19,7 +23,17 @@ __global__ void k_weights(FinParams p) {
   const uint8_t* va = p.valid + (size_t)a * p.ld;
   const uint8_t* vb = p.valid + (size_t)b * p.ld;
   int cnt = 0;
-  for (int i = threadIdx.x; i < p.M; i += blockDim.x) cnt += (va[i] && vb[i]) ? 1 : 0;
+  const int vec = p.ld % 16 == 0 ? p.M : 0;  // bytes of 0 or 1
+  for (int i = 16 * threadIdx.x; i < vec; i += 16 * blockDim.x) {
+    const uint4 x = *reinterpret_cast<const uint4*>(va + i), y = *reinterpret_cast<const uint4*>(vb + i);
+    const uint32_t w[4] = {x.x & y.x, x.y & y.y, x.z & y.z, x.w & y.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int n = p.M - i - 4 * q;  // blocks of the integration in this word
+      cnt += __popc(n >= 4 ? w[q] : n > 0 ? w[q] & ((1u << (8 * n)) - 1u) : 0u);
+    }
+  }
+  for (int i = vec + threadIdx.x; i < p.M; i += blockDim.x) cnt += va[i] & vb[i];
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
   __shared__ int ws[32];
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = cnt;
@@ -37,63 +51,115 @@ cudaError_t launch_weights(const FinParams& p, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-__global__ void k_finalize(FinParams p) {
+// 1 / (W N) of a baseline times `unscale`: in FP64, which this GPU runs at a
+// 64th of its FP32 rate, so one thread of a CTA forms it, not every element.
+__device__ __forceinline__ float fin_scale(const FinParams& p, int bl, float unscale) {
+  const int w = p.wcount[bl];
+  return w > 0 ? (float)((double)unscale / ((double)w * (double)p.N)) : 0.f;
+}
+
+// Partial sums [KZ][nbl][G][nchan] -> out.  A CTA takes elements of one
+// baseline (blockIdx.y), shared by KG groups of 256 / KG threads: group q adds
+// partials q, q + KG, ... and the groups' sums are added in order.  Up to 8
+// partials (KG = 1): one streaming pass of eight loads in flight per thread,
+// bound by HBM (2080 baselines x 131072 values, one partial, 4.4 GB: 5.5 ms
+// with an FP64 quotient per element, 0.62 ms now).  Above, the sum of one
+// element is a long chain of loads and the output small (a two-station scan
+// has 768 values of 456 partials: 66 us as one chain, 9.5 us now), so sixteen
+// groups share it.
+template <int KG>
+__global__ void __launch_bounds__(256) k_finalize(FinParams p) {
+  constexpr int EL = 256 / KG, PER = KG == 1 ? 8 : 1;  // a thread takes PER elements, EL apart
+  const int bl = blockIdx.y;
   const size_t per = (size_t)p.G * p.nchan;
   const size_t total = (size_t)nbl_of(p.S) * per;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  __shared__ float s_sc;
+  __shared__ float2 s_sum[KG > 1 ? 256 : 1];
+  if (threadIdx.x == 0) s_sc = fin_scale(p, bl, p.unscale);
   const bool failed = p.err && *p.err != 0;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
-    const int bl = (int)(e / per);
-    float2 v = make_float2(0.f, 0.f);
-    for (int kz = 0; kz < p.KZ; ++kz) {
-      const float2 x = p.part[(size_t)kz * total + e];
-      v.x += x.x;
-      v.y += x.y;
-    }
-    const int w = p.wcount[bl];
-    const float sc = w > 0 ? (float)((double)p.unscale / ((double)w * (double)p.N)) : 0.f;
-    p.out[e] = failed ? make_float2(__int_as_float(0x7fc00000), __int_as_float(0x7fc00000))
-                      : make_float2(v.x * sc, v.y * sc);
+  const int q = threadIdx.x / EL;
+  const size_t k = (size_t)blockIdx.x * EL * PER + threadIdx.x % EL;
+  float2 v[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) v[u] = make_float2(0.f, 0.f);
+#pragma unroll(KG > 1 ? 8 : 1)
+  for (int kz = q; kz < p.KZ; kz += KG) {
+    const float2* src = p.part + (size_t)kz * total + (size_t)bl * per + k;
+    float2 x[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) x[u] = k + u * EL < per ? __ldcs(src + u * EL) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) v[u] = make_float2(v[u].x + x[u].x, v[u].y + x[u].y);
   }
+  if constexpr (KG > 1) s_sum[threadIdx.x] = v[0];
+  __syncthreads();
+  if (q != 0) return;
+  if constexpr (KG > 1) {
+#pragma unroll
+    for (int g = 1; g < KG; ++g) {
+      const float2 x = s_sum[g * EL + threadIdx.x];
+      v[0].x += x.x;
+      v[0].y += x.y;
+    }
+  }
+  const float nan = __int_as_float(0x7fc00000);
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+    if (k + u * EL < per)
+      p.out[(size_t)bl * per + k + u * EL] = failed ? make_float2(nan, nan) : make_float2(v[u].x * s_sc, v[u].y * s_sc);
 }
 
 cudaError_t launch_finalize(const FinParams& p, cudaStream_t s) {
-  const size_t total = (size_t)nbl_of(p.S) * p.G * p.nchan;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  if (blocks < 1) blocks = 1;
-  k_finalize<<<blocks, 256, 0, s>>>(p);
+  const size_t per = (size_t)p.G * p.nchan;
+  if (p.KZ > 8)
+    k_finalize<16><<<dim3((unsigned)((per + 15) / 16), nbl_of(p.S)), 256, 0, s>>>(p);
+  else
+    k_finalize<1><<<dim3((unsigned)((per + 2047) / 2048), nbl_of(p.S)), 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
-// Tensor-core partial sums are laid out [KZ][G][nchan][nbl] (baseline
-// fastest, as the X kernel's epilogue writes them).
-__global__ void k_finalize_tc(FinParams p, float unscale) {
+// Tensor-core partial sums are laid out [G][nchan][nbl] (baseline fastest, as
+// the X kernel's epilogue adds them), the output is [nbl][G][nchan]: 32 x 32
+// values are turned through shared memory so that both the reads and the
+// writes are 256-byte runs.  Bound by HBM: 2080 baselines x 131072 channels
+// (2.2 GB each way) took 6.0 ms with 8-byte reads 16 KB apart and an FP64
+// quotient per value, 0.64 ms now, 6.8 TB/s.
+constexpr int kTurn = 32;
+__device__ __forceinline__ void load_turn(const FinParams& p, size_t gk0, size_t per, int bl0, int nbl,
+                                          float2 (&tile)[kTurn][kTurn + 1]) {
+#pragma unroll
+  for (int r = 0; r < kTurn; r += 8) {
+    const size_t gk = gk0 + r + threadIdx.y;
+    const int bl = bl0 + threadIdx.x;
+    if (gk < per && bl < nbl) tile[r + threadIdx.y][threadIdx.x] = __ldcs(p.part + gk * nbl + bl);
+  }
+}
+
+__global__ void __launch_bounds__(256) k_finalize_tc(FinParams p, float unscale) {
+  __shared__ float2 tile[kTurn][kTurn + 1];
+  __shared__ float s_sc[kTurn];
   const int nbl = nbl_of(p.S);
   const size_t per = (size_t)p.G * p.nchan;
-  const size_t total = (size_t)nbl * per;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
-    const int bl = (int)(e / per);
-    const size_t gk = e - (size_t)bl * per;  // g * nchan + k
-    float2 v = make_float2(0.f, 0.f);
-    for (int kz = 0; kz < p.KZ; ++kz) {
-      const float2 x = p.part[((size_t)kz * per + gk) * nbl + bl];
-      v.x += x.x;
-      v.y += x.y;
+  const int bl0 = blockIdx.y * kTurn;
+  const size_t gk0 = (size_t)blockIdx.x * kTurn;
+  if (threadIdx.y == 0) s_sc[threadIdx.x] = bl0 + threadIdx.x < nbl ? fin_scale(p, bl0 + threadIdx.x, unscale) : 0.f;
+  load_turn(p, gk0, per, bl0, nbl, tile);
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kTurn; r += 8) {
+    const int row = r + threadIdx.y;
+    const size_t gk = gk0 + threadIdx.x;
+    if (gk < per && bl0 + row < nbl) {
+      const float2 v = tile[threadIdx.x][row];
+      p.out[(size_t)(bl0 + row) * per + gk] = make_float2(v.x * s_sc[row], v.y * s_sc[row]);
     }
-    const int w = p.wcount[bl];
-    const float sc = w > 0 ? (float)((double)unscale / ((double)w * (double)p.N)) : 0.f;
-    p.out[e] = make_float2(v.x * sc, v.y * sc);
   }
 }
 
 cudaError_t launch_finalize_tc(const FinParams& p, float unscale, cudaStream_t s) {
-  const size_t total = (size_t)nbl_of(p.S) * p.G * p.nchan;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  if (blocks < 1) blocks = 1;
-  k_finalize_tc<<<blocks, 256, 0, s>>>(p, unscale);
+  const size_t per = (size_t)p.G * p.nchan;
+  const int nbl = nbl_of(p.S);
+  k_finalize_tc<<<dim3((unsigned)((per + kTurn - 1) / kTurn), (nbl + kTurn - 1) / kTurn), dim3(kTurn, 8), 0, s>>>(p, unscale);
   return cudaGetLastError();
 }
 
@@ -101,31 +167,39 @@ cudaError_t launch_finalize_tc(const FinParams& p, float unscale, cudaStream_t s
 // v = pol * S + station per subband, so V_ab^pq is the virtual product
 // P[p S + a][q S + b] when p S + a <= q S + b and its conjugate otherwise
 // (for a = b and pq = 10: the conjugate of the 01 product).
+__device__ __forceinline__ int cross_source(int S, int a, int b, int pq, bool& flip) {
+  int v1 = (pq >> 1) * S + a, v2 = (pq & 1) * S + b;
+  flip = v1 > v2;
+  if (flip) {
+    const int t = v1;
+    v1 = v2;
+    v2 = t;
+  }
+  return bl_index(v1, v2, 2 * S);
+}
+
+// A CTA takes one baseline (blockIdx.y) and a run of (subband, hand, channel)
+// values.
 template <bool TC>
-__global__ void k_finalize_cross(FinParams p, float unscale) {
-  const int S = p.S, S2 = 2 * S, nsub = p.G, nch = p.nchan;
-  const int nblv = nbl_of(S2);
-  const size_t total = (size_t)nbl_of(S) * nsub * 4 * nch;
-  const size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += stride) {
-    const int k = (int)(e % nch);
-    size_t r = e / nch;
-    const int pq = (int)(r & 3);
-    r >>= 2;
-    const int sb = (int)(r % nsub);
-    const int bl = (int)(r / nsub);
-    int a = 0, q = bl;
-    while (q >= S - a) { q -= S - a; ++a; }
-    const int b = a + q;
-    int v1 = (pq >> 1) * S + a, v2 = (pq & 1) * S + b;
-    const bool flip = v1 > v2;
-    if (flip) {
-      const int t = v1;
-      v1 = v2;
-      v2 = t;
-    }
-    const int blv = bl_index(v1, v2, S2);
+__global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unscale) {
+  const int S = p.S, nsub = p.G, nch = p.nchan;
+  const int nblv = nbl_of(2 * S);
+  const int bl = blockIdx.y;
+  __shared__ float s_sc;
+  if (threadIdx.x == 0) s_sc = fin_scale(p, bl, unscale);
+  __syncthreads();
+  int a = 0, q = bl;
+  while (q >= S - a) { q -= S - a; ++a; }
+  const int b = a + q;
+  const int per = nsub * 4 * nch;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < per; e += gridDim.x * blockDim.x) {
+    const int k = e & (nch - 1);  // a power of two of channels
+    const int r = e / nch;
+    const int pq = r & 3, sb = r >> 2;
+    bool flip;
+    const int blv = cross_source(S, a, b, pq, flip);
     float2 v = make_float2(0.f, 0.f);
+#pragma unroll 4
     for (int kz = 0; kz < p.KZ; ++kz) {
       const float2 x = TC ? p.part[(((size_t)kz * nsub + sb) * nch + k) * nblv + blv]
                           : p.part[(((size_t)kz * nblv + blv) * nsub + sb) * nch + k];
@@ -133,21 +207,17 @@ __global__ void k_finalize_cross(FinParams p, float unscale) {
       v.y += x.y;
     }
     if (flip) v.y = -v.y;
-    const int w = p.wcount[bl];
-    const float sc = w > 0 ? (float)((double)unscale / ((double)w * (double)p.N)) : 0.f;
-    p.out[e] = make_float2(v.x * sc, v.y * sc);
+    p.out[(size_t)bl * per + e] = make_float2(v.x * s_sc, v.y * s_sc);
   }
 }
 
 cudaError_t launch_finalize_cross(const FinParams& p, bool tc, float unscale, cudaStream_t s) {
-  const size_t total = (size_t)nbl_of(p.S) * p.G * 4 * p.nchan;
-  int blocks = (int)((total + 255) / 256);
-  if (blocks > 152 * 16) blocks = 152 * 16;
-  if (blocks < 1) blocks = 1;
+  const int per = p.G * 4 * p.nchan;
+  const dim3 grid((per + 1023) / 1024, nbl_of(p.S));
   if (tc)
-    k_finalize_cross<true><<<blocks, 256, 0, s>>>(p, unscale);
+    k_finalize_cross<true><<<grid, 256, 0, s>>>(p, unscale);
   else
-    k_finalize_cross<false><<<blocks, 256, 0, s>>>(p, unscale);
+    k_finalize_cross<false><<<grid, 256, 0, s>>>(p, unscale);
   return cudaGetLastError();
 }
 
