@@ -4,28 +4,31 @@
 // a chunk:  V_ab[k] += X_a[k] conj(X_b[k]) for every baseline a <= b
 // (autocorrelations included, parallel hands only).
 //
-// One thread owns one channel of one stream and a TA x TA tile of baselines
-// (a diagonal tile keeps only a <= b), so each loaded spectrum value is used
-// TA times from registers.  The blocks of a chunk are split into KZ ranges;
-// each range sums at most 256 blocks in registers and then adds that partial
-// into its own FP32 accumulator slice part[kz], in a fixed order, so results
-// are deterministic and the FP32 sums stay short (hierarchical accumulation).
+// A lane owns one channel of one stream and all baselines of a tile of TS
+// stations (a <= b), or of two different tiles (TS x TS), in registers, so
+// each value read from shared memory meets TS others.  Up to 12 stations are
+// one tile (k_xmac); more are split into tiles of 5 to 8, and the warps of a
+// CTA hold up to 12 tile pairs of the same 32 channels, so that a station's
+// values are fetched once for all of them (k_xpairs).  The blocks of a chunk
+// are split into KZ ranges; each range sums at most 256 blocks in registers
+// and then adds that partial into its own FP32 accumulator slice part[kz], one
+// add per element and launch, so results are deterministic and the FP32 sums
+// stay short (hierarchical accumulation).
 #include "corr_internal.cuh"
 
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
-#include <type_traits>
 #include <cudaTypedefs.h>
+
+#include <string.h>
+
+#include <algorithm>
+#include <type_traits>
 
 namespace corr {
 
-constexpr int kXT = 128;  // threads per CTA (channels)
-
-// 16-byte asynchronous copy to shared memory; src_bytes = 0 writes zeros.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes));
-}
+namespace {
 
 // acc + x conj(y) on packed FP32 pairs: acc + x (y.x, y.x) + xr (y.y, y.y)
 // with xr = (x.y, -x.x), formed once per loaded value: two f32x2 fused
@@ -39,532 +42,590 @@ __device__ __forceinline__ float2 rot_conj(float2 x) { return __fmul2_rn(make_fl
 __device__ __forceinline__ float2 cmac_auto(float2 acc, float2 x) { return __ffma2_rn(x, x, acc); }
 __device__ __forceinline__ float2 auto_value(float2 acc) { return make_float2(acc.x + acc.y, 0.f); }
 
-// The tile pairs of one 128-channel tile are consecutive CTAs (blockIdx.x
-// = channel tile x pairs + pair), so the pairs that read the same stations'
-// spectra run side by side and all but the first read come from L2.  The
-// diagonal pairs (DIAG) and the off-diagonal ones are separate launches.
-// The 2 x 8 stations' values of each block reach shared memory through a
-// cp.async ring of kStagesT blocks, so that many blocks' loads are in flight
-// without registers (the accumulators take 128 of them).
-// First tile row of part `part` of `npart` for a triangular tile: the parts
-// get about equal numbers of baselines (row i holds TA - i of them).
-__host__ __device__ constexpr int tri_split(int TA, int npart, int part) {
-  if (part <= 0) return 0;
-  if (part >= npart) return TA;
-  int acc = 0, i = 0;
-  const int total = TA * (TA + 1) / 2;
-  while (i < TA && 2 * npart * (acc + (TA - i)) <= 2 * total * part + npart * (TA - i)) {
-    acc += TA - i;
-    ++i;
-  }
-  return i;
-}
-
-constexpr int kStagesT = 4;
-
-// Two threads per channel: thread part 0 takes tile rows [0, SPLIT) and
-// part 1 rows [SPLIT, TA) (half the baselines each), so a thread holds 32
-// accumulators instead of 64 and an SM runs twice the warps.
-template <int TA, bool DIAG>
-__global__ void __launch_bounds__(2 * kXT) k_xmac(XParams p, int ntile) {
-  extern __shared__ __align__(16) unsigned char xt_raw[];
-  constexpr int NT = DIAG ? 1 : 2;                 // station tiles per block
-  float2* ring = reinterpret_cast<float2*>(xt_raw);  // [kStagesT][NT][TA][kXT]
-  const int npo = DIAG ? ntile : ntile * (ntile - 1) / 2;  // pairs of this launch
-  const int pidx = blockIdx.x % npo;
-  const int k0 = (blockIdx.x / npo) * kXT;
-  const int lane = threadIdx.x % kXT;
-  const int part = threadIdx.x / kXT;
-  const int k = k0 + lane;
-  const int g = blockIdx.y;
-  const int kz = blockIdx.z;
-  int ta = pidx, tb = pidx;
-  if (!DIAG) {  // off-diagonal pair pidx in row-major order over ta < tb
-    int q = pidx;
-    ta = 0;
-    while (q >= ntile - 1 - ta) { q -= ntile - 1 - ta; ++ta; }
-    tb = ta + 1 + q;
-  }
-  const int S = p.S;
-  const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
-  const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
-  if (b_hi <= b_lo) return;
-  const int nb = b_hi - b_lo;
-  constexpr int stage_elems = NT * TA * kXT;
-  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-  const size_t sstride = (size_t)p.nchan;
-
-  // copies of block b_lo + q into slot q % kStagesT: NT x TA rows of 128
-  // channels, 64 pieces of 16 bytes each; rows beyond S and channels beyond
-  // nchan are zero-filled
-  auto issue = [&](int q) {
-    if (q < nb) {
-      const int slot = q % kStagesT;
-      const int b = b_lo + q;
-      for (int e = threadIdx.x; e < NT * TA * 64; e += 2 * kXT) {
-        const int piece = e & 63;
-        const int row = e >> 6;                     // (tile, station in tile)
-        const int st = ((row >= TA) ? tb : ta) * TA + (row % TA);
-        const int ch = k0 + piece * 2;
-        const bool in = st < S && ch < p.nchan;
-        const float2* src = p.spec + ((size_t)g * p.CB + b) * (size_t)S * sstride + (size_t)(in ? st : 0) * sstride +
-                            (in ? ch : 0);
-        const uint32_t dst = ring_s + (uint32_t)((slot * stage_elems + row * kXT + piece * 2) * 8);
-        cp_async16(dst, src, in ? 16 : 0);
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-
-  auto run = [&](auto I0c, auto I1c) {
-    constexpr int I0 = decltype(I0c)::value, I1 = decltype(I1c)::value;
-    float2 acc[TA][TA];
-#pragma unroll
-    for (int i = I0; i < I1; ++i)
-#pragma unroll
-      for (int j = 0; j < TA; ++j) acc[i][j] = make_float2(0.f, 0.f);
-
-    for (int q = 0; q < kStagesT - 1; ++q) issue(q);
-    for (int q = 0; q < nb; ++q) {
-      issue(q + kStagesT - 1);
-      asm volatile("cp.async.wait_group %0;" ::"n"(kStagesT - 1) : "memory");
-      __syncthreads();
-      const float2* st = ring + (q % kStagesT) * stage_elems + lane;
-      float2 a[TA], b[TA];
-#pragma unroll
-      for (int i = I0; i < (DIAG ? TA : I1); ++i) a[i] = st[i * kXT];
-      if (!DIAG) {
-#pragma unroll
-        for (int i = 0; i < TA; ++i) b[i] = st[(TA + i) * kXT];
-      }
-#pragma unroll
-      for (int i = I0; i < I1; ++i) {
-        const float2 ar = rot_conj(a[i]);
-#pragma unroll
-        for (int j = DIAG ? i : 0; j < TA; ++j)
-          acc[i][j] = (DIAG && j == i) ? cmac_auto(acc[i][j], a[i])
-                                       : cmac_conj(acc[i][j], a[i], ar, DIAG ? a[j] : b[j]);  // X_a conj(X_b)
-      }
-      __syncthreads();
-    }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    if (k >= p.nchan) return;
-    const int nbl = nbl_of(S);
-#pragma unroll
-    for (int i = I0; i < I1; ++i)
-#pragma unroll
-      for (int j = DIAG ? i : 0; j < TA; ++j) {
-        const int sa = ta * TA + i, sb = tb * TA + j;
-        if (sa < S && sb < S) {
-          float2* dst = p.part + (((size_t)kz * nbl + bl_index(sa, sb, S)) * p.G + g) * sstride + k;
-          const float2 x = (DIAG && j == i) ? auto_value(acc[i][j]) : acc[i][j];
-          float2 v = *dst;
-          v.x += x.x;
-          v.y += x.y;
-          *dst = v;
-        }
-      }
-  };
-  constexpr int SPLIT = DIAG ? tri_split(TA, 2, 1) : TA / 2;
-  if (part == 0)
-    run(std::integral_constant<int, 0>{}, std::integral_constant<int, SPLIT>{});
-  else
-    run(std::integral_constant<int, SPLIT>{}, std::integral_constant<int, TA>{});
-}
-
-// For S <= 12 (one triangular tile of baselines per channel) the spectra
-// reach the threads through a shared-memory ring filled by cp.async, so the
-// number of bytes in flight no longer depends on how many registers the
-// accumulators take: kStagesX stages of kNB blocks x S stations x 128
-// channels, one CTA per (128-channel tile, stream, block range).
-constexpr int kNB = 2;       // blocks per stage
-constexpr int kStagesX = 4;  // ring depth
-
-
-template <int TA>
-__global__ void __launch_bounds__(kXT) k_xmac_ring(XParams p) {
-  extern __shared__ __align__(16) unsigned char xs_raw[];
-  float2* ring = reinterpret_cast<float2*>(xs_raw);  // [kStagesX][kNB][S][kXT]
-  const int tid = threadIdx.x;
-  const int k0 = blockIdx.x * kXT;
-  const int k = k0 + tid;
-  const int g = blockIdx.y;
-  const int kz = blockIdx.z;
-  const int S = p.S;
-  const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
-  const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
-  if (b_hi <= b_lo) return;
-  const int nst = (b_hi - b_lo + kNB - 1) / kNB;  // stages of this CTA
-  const int stage_elems = kNB * S * kXT;
-  const uint32_t ring_s = (uint32_t)__cvta_generic_to_shared(ring);
-
-  // issue the copies of stage q (blocks b_lo + q*kNB ...) into ring slot q % kStagesX
-  auto issue = [&](int q) {
-    if (q < nst) {
-      const int slot = q % kStagesX;
-      const int chunks = kNB * S * (kXT * 8 / 16);  // 16-byte pieces
-      for (int c = tid; c < chunks; c += kXT) {
-        const int row = c >> 6;                    // (block-in-stage, station), 64 pieces per row
-        const int piece = c & 63;
-        const int bi = row / S;
-        const int st = row - bi * S;
-        const int b = b_lo + q * kNB + bi;
-        const int ch = k0 + piece * 2;
-        const bool in = b < b_hi && ch < p.nchan;
-        const float2* src = p.spec + ((size_t)g * p.CB + (in ? b : b_lo)) * (size_t)S * p.nchan +
-                            (size_t)st * p.nchan + (in ? ch : 0);
-        const uint32_t dst = ring_s + (uint32_t)(((slot * kNB + bi) * S + st) * kXT + piece * 2) * 8u;
-        cp_async16(dst, src, in ? 16 : 0);
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-
-  float2 acc[TA][TA];
-#pragma unroll
-  for (int i = 0; i < TA; ++i)
-#pragma unroll
-    for (int j = 0; j < TA; ++j) acc[i][j] = make_float2(0.f, 0.f);
-
-#pragma unroll
-  for (int q = 0; q < kStagesX - 1; ++q) issue(q);
-  for (int q = 0; q < nst; ++q) {
-    issue(q + kStagesX - 1);
-    asm volatile("cp.async.wait_group %0;" ::"n"(kStagesX - 1) : "memory");
-    __syncthreads();
-    const float2* st = ring + (q % kStagesX) * stage_elems;
-#pragma unroll
-    for (int bi = 0; bi < kNB; ++bi) {
-      float2 a[TA];
-#pragma unroll
-      for (int i = 0; i < TA; ++i) a[i] = i < S ? st[(bi * S + i) * kXT + tid] : make_float2(0.f, 0.f);
-#pragma unroll
-      for (int i = 0; i < TA; ++i) {
-        const float2 ar = rot_conj(a[i]);
-#pragma unroll
-        for (int j = i; j < TA; ++j) acc[i][j] = j == i ? cmac_auto(acc[i][j], a[i]) : cmac_conj(acc[i][j], a[i], ar, a[j]);
-      }
-    }
-    __syncthreads();
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  if (k >= p.nchan) return;
-  const int nbl = nbl_of(S);
-#pragma unroll
-  for (int i = 0; i < TA; ++i)
-#pragma unroll
-    for (int j = i; j < TA; ++j)
-      if (i < S && j < S) {
-        // one add per element per launch: deterministic fire-and-forget reduction
-        float* dst = reinterpret_cast<float*>(p.part + (((size_t)kz * nbl + bl_index(i, j, S)) * p.G + g) *
-                                                           (size_t)p.nchan + k);
-        if (j == i) {
-          atomicAdd(dst, auto_value(acc[i][j]).x);
-        } else {
-          atomicAdd(dst, acc[i][j].x);
-          atomicAdd(dst + 1, acc[i][j].y);
-        }
-      }
-}
-
-// The same X step with the ring filled by the tensor memory accelerator: one
-// 2-D tensor copy per stage (box: 128 channels x (kNB blocks x S stations))
-// instead of 16-byte copies from every thread, so the bytes in flight are not
-// limited by per-thread outstanding requests.  Thread 0 issues the copies; an
-// mbarrier with a transaction count per ring slot signals arrival; every wait
-// is bounded (timeout -> *err, the CTA stops issuing and returns).
 constexpr long long kXDrainLimit = 1LL << 26;  // spins per wait while draining after an abort
+constexpr int kMaxStages = 8;                  // ring depth
+constexpr int kGroupWarps = 12;                // tile pairs per CTA (168 registers a thread at TS = 8)
+constexpr int kGroupTiles = 8;                 // station tiles a CTA stages
+constexpr int kOneTile = 12;                   // stations held as one tile
+constexpr int kMaxXStations = 2 * kMaxStations;
+
+// What one CTA of the many-station form works on: the station tiles that it
+// stages, and per warp the places in that list of its tile pair (equal: the
+// baselines inside a tile).
+struct XGroup {
+  uint8_t nwarp, ntile;
+  uint8_t tile[kGroupTiles];
+  uint8_t wa[kGroupWarps], wb[kGroupWarps];
+};
+constexpr int kMaxTiles = kMaxXStations / 8;  // 8 is the tile above 64 stations
+constexpr int kMaxGroups = 2 * (kMaxTiles * (kMaxTiles + 1) / 2) / kGroupWarps;
+struct XGroups {
+  int n;
+  XGroup g[kMaxGroups];
+};
 
 __device__ __forceinline__ uint32_t xs_u32(const void* ptr) { return (uint32_t)__cvta_generic_to_shared(ptr); }
 
-// Two threads per channel (256 per CTA): thread part 0 owns tile rows
-// [0, SPLIT), part 1 rows [SPLIT, TA) -- about half the baselines each --
-// so twice the warps share one ring of spectra.
-constexpr int kXThreadsT = 2 * kXT;
-
-// Bytes per spectrum value of each input kind: FP32 complex, FP16 complex
-// (half2), E4M3 complex (two bytes, Re low).
-// Blocks per ring stage: 2 of FP32, 4 of FP16, 8 of E4M3 values, so that a
-// stage (and the bytes in flight per CTA) is the same size for every kind.
-template <int IN> struct SpecElem {
-  static constexpr int bytes = IN == 0 ? 8 : (IN == 1 ? 4 : 2);
-  static constexpr int nb = kNB * 8 / bytes;
-};
-
-// One spectrum value from the ring as FP32 (the FP16 / E4M3 values carry
-// X * 2^-sigma; the normalisation takes the 2^(2 sigma) back out).
+// One spectrum value of lane `i` from the ring as FP32 (the FP16 / E4M3
+// values carry X * 2^-sigma; the normalisation takes the 2^(2 sigma) back out).
 template <int IN>
-__device__ __forceinline__ float2 ring_value(const unsigned char* st, int idx) {
+__device__ __forceinline__ float2 ring_value(const unsigned char* st, int i) {
   if constexpr (IN == 0) {
-    return reinterpret_cast<const float2*>(st)[idx];
+    return reinterpret_cast<const float2*>(st)[i];
   } else if constexpr (IN == 1) {
-    return __half22float2(reinterpret_cast<const __half2*>(st)[idx]);
+    return __half22float2(reinterpret_cast<const __half2*>(st)[i]);
   } else {
-    const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2(reinterpret_cast<const __nv_fp8x2_storage_t*>(st)[idx], __NV_E4M3);
+    const __half2_raw h = __nv_cvt_fp8x2_to_halfraw2(reinterpret_cast<const __nv_fp8x2_storage_t*>(st)[i], __NV_E4M3);
     return __half22float2(__half2(h));
   }
 }
 
-template <int TA, int IN>
-__global__ void __launch_bounds__(kXThreadsT) k_xmac_tma(const __grid_constant__ CUtensorMap tmap, XParams p) {
-  extern __shared__ __align__(1024) unsigned char xs_tma_raw[];
-  const uint32_t raw = xs_u32(xs_tma_raw);
-  constexpr int EB = SpecElem<IN>::bytes;
-  constexpr int NB = SpecElem<IN>::nb;
-  unsigned char* ring = xs_tma_raw + (((raw + 1023u) & ~1023u) - raw);  // [kStagesX][NB*S][kXT] values
-  __shared__ __align__(8) uint64_t full[kStagesX];
-  __shared__ int s_abort;
-  const int tid = threadIdx.x;
-  const int lane_ch = tid % kXT;
-  const int part = tid / kXT;
-  const int k0 = blockIdx.x * kXT;
-  const int k = k0 + lane_ch;
-  const int g = blockIdx.y;
-  const int kz = blockIdx.z;
-  const int S = p.S;
+constexpr int spec_bytes(int in) { return in == 0 ? 8 : (in == 1 ? 4 : 2); }  // per complex value
+
+// Bounded wait for a phase of an mbarrier: gives up when the CTA's abort flag
+// is set or after `limit` polls.
+__device__ __forceinline__ bool ring_poll(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+               : "=r"(ok)
+               : "r"(xs_u32(bar)), "r"(parity)
+               : "memory");
+  return ok;
+}
+__device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+  for (long long it = 0; it < limit; ++it) {
+    if (ring_poll(bar, parity)) return true;
+    if ((it & 1023) == 1023 && *abort_flag) return false;
+  }
+  return false;
+}
+
+// A ring of shared-memory stages filled by tensor copies.  Each stage has an
+// mbarrier `full` (the copies' byte count) and `empty` (one arrival per
+// reading warp).  At its iteration q one of the warps, each in its turn, refills
+// the slot of stage q - 2: issuing copies holds a warp up for most of a
+// thousand cycles, and waiting for the slowest reader of stage q - 1 would
+// hold up the whole CTA (64 stations x 8 streams x 4096 channels x 128 blocks:
+// 1.58 ms; warp 0 refilling each time 1.69, slot q - 1 instead 2.33).
+struct Ring {
+  uint64_t *full, *empty;
+  volatile int *abort_flag, *issued;  // `issued`: stages whose copies were issued, in order
+  int stages;
+  long long limit;
+
+  __device__ __forceinline__ void init(int readers) {
+    if (threadIdx.x == 0) {
+      for (int i = 0; i < stages; ++i) {
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(xs_u32(&full[i])));
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(xs_u32(&empty[i])), "r"(readers));
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      *abort_flag = 0;
+      *issued = 0;
+    }
+    __syncthreads();
+  }
+  // at stage q, held in `slot` with parity `phase`: the place of stage q - 2, once every warp has read it (-1: gave up)
+  __device__ __forceinline__ int reclaim(int slot, uint32_t phase) const {
+    const int old = slot >= 2 ? slot - 2 : slot - 2 + stages;
+    if (ring_wait(&empty[old], old > slot ? phase ^ 1 : phase, abort_flag, limit)) return old;
+    *abort_flag = 1;
+    return -1;
+  }
+  // a warp has read stage slot `slot`
+  __device__ __forceinline__ void release(int slot) const {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0)
+      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(xs_u32(&empty[slot])) : "memory");
+  }
+  // After an abort, with every warp of the CTA past its last issue: let the
+  // copies in flight land before the CTA's shared memory goes away.
+  __device__ __forceinline__ void drain(int* err) const {
+    const int n = *issued;
+    for (int q = n > stages ? n - stages : 0; q < n; ++q)
+      for (long long it = 0; it < kXDrainLimit; ++it)
+        if (ring_poll(&full[q % stages], (uint32_t)((q / stages) & 1))) break;
+    if (err) atomicExch(err, 1);
+  }
+};
+
+// The accumulators of one tile pair and their update by one block: `ra` and
+// `rb` point at the tiles' staged rows of this lane's channel.
+template <int TS, int IN, bool DIAG>
+__device__ __forceinline__ void tile_block(float2 (&acc)[TS][TS], const unsigned char* ra, const unsigned char* rb,
+                                           int row_bytes) {
+  float2 b[TS];
+#pragma unroll
+  for (int j = 0; j < TS; ++j) b[j] = ring_value<IN>(rb + j * row_bytes, 0);
+#pragma unroll
+  for (int i = 0; i < TS; ++i) {
+    const float2 a = DIAG ? b[i] : ring_value<IN>(ra + i * row_bytes, 0);
+    const float2 ar = rot_conj(a);
+#pragma unroll
+    for (int j = DIAG ? i : 0; j < TS; ++j)
+      acc[i][j] = (DIAG && j == i) ? cmac_auto(acc[i][j], a) : cmac_conj(acc[i][j], a, ar, b[j]);
+  }
+}
+
+// Add a tile pair's sums to the partial sums: part[baseline * row] of this
+// lane's stream and channel, one add per element and launch.
+template <int TS, bool DIAG>
+__device__ __forceinline__ void add_tile(const float2 (&acc)[TS][TS], float2* part, size_t row, int a0, int b0, int S) {
+#pragma unroll
+  for (int i = 0; i < TS; ++i)
+#pragma unroll
+    for (int j = DIAG ? i : 0; j < TS; ++j)
+      if (a0 + i < S && b0 + j < S) {
+        float2* dst = part + (size_t)bl_index(a0 + i, b0 + j, S) * row;
+        if (DIAG && j == i)
+          atomicAdd(&dst->x, auto_value(acc[i][j]).x);
+        else
+          asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(acc[i][j].x), "f"(acc[i][j].y) : "memory");
+      }
+}
+
+// CTAs per SM of the one-tile form: TS (TS + 1) accumulators a lane.
+constexpr int one_tile_ctas(int TS) { return TS <= 5 ? 6 : TS <= 8 ? 4 : TS <= 11 ? 3 : 2; }
+
+struct XShape {
+  int nb;          // blocks per ring stage
+  int nst;         // ring stages
+  int cg;          // channel groups of 32, one warp each (k_xmac)
+  int pitch;       // channels per staged row: 32 cg, or nchan if fewer
+  int tile_bytes;  // nb blocks of one tile, rounded up to the copies' 128-byte alignment
+  int stage_bytes;
+};
+
+// Up to 12 stations: one CTA of cg warps takes 32 cg channels of stream
+// blockIdx.y and block range blockIdx.z.  Its ring's stages hold nb blocks of
+// all stations, [block][station][channel], each filled by one tensor copy.
+// Every wait is bounded (timeout -> *err; the CTA stops and lets its copies
+// land).
+//
+// FP32 spectra: bound by HBM.  FP16 / E4M3 spectra: by the FMA pipe and the
+// register moves of its paired operands (one lane for all 55 baselines of ten
+// stations reads 10 values a block, where two lanes with half the baselines
+// each read 17).  A stage takes as many blocks as four of them fit: a copy
+// costs the copy engine about 13 cycles per row of up to 1 KB on top of about
+// 60, and a stage its warps' waits.  Ten stations x 16 streams x 1024
+// channels, 819 blocks: FP32 167 us (6.4 TB/s), FP16 129, E4M3 123 us; with two
+// lanes a channel and two barriers a stage 178, 151 and 150 us.
+template <int TS, int IN>
+__global__ void __launch_bounds__(128, one_tile_ctas(TS))
+k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams p, const XShape sh) {
+  extern __shared__ __align__(128) unsigned char ring_raw[];
+  unsigned char* data = ring_raw + ((128u - (xs_u32(ring_raw) & 127u)) & 127u);
+  __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
+  __shared__ volatile int s_abort, s_issued;
+  constexpr int EB = spec_bytes(IN);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int k0 = blockIdx.x * 32 * sh.cg;
+  const int k = k0 + threadIdx.x;
+  const int g = blockIdx.y, kz = blockIdx.z;
   const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
   const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
   if (b_hi <= b_lo) return;
-  const int nst = (b_hi - b_lo + NB - 1) / NB;
-  const int stage_elems = NB * S * kXT;
-  const uint32_t stage_bytes = (uint32_t)stage_elems * EB;
-  if (tid == 0) {
-    for (int i = 0; i < kStagesX; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(xs_u32(&full[i])));
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    s_abort = 0;
-  }
-  __syncthreads();
-
-  auto issue = [&](int q) {
-    if (q >= nst) return;
-    const int slot = q % kStagesX;
-    const int row = (g * p.CB + b_lo + q * NB) * S;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xs_u32(&full[slot])),
-                 "r"(stage_bytes)
+  const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
+  const int row_bytes = sh.pitch * EB;
+  Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
+  ring.init(sh.cg);
+  auto issue = [&](int q, int slot) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xs_u32(&s_full[slot])),
+                 "r"(sh.nb * TS * row_bytes)
                  : "memory");
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            xs_u32(ring + (size_t)slot * stage_bytes)),
-        "l"(reinterpret_cast<uint64_t>(&tmap)), "r"(2 * k0), "r"(row), "r"(xs_u32(&full[slot]))
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(xs_u32(data) + (uint32_t)(slot * sh.stage_bytes)),
+        "l"(reinterpret_cast<uint64_t>(&tmap)), "r"(2 * k0), "r"(0), "r"(g * p.CB + b_lo + q * sh.nb),
+        "r"(xs_u32(&s_full[slot]))
         : "memory");
+    s_issued = q + 1;
   };
+  if (threadIdx.x == 0)
+    for (int q = 0; q < sh.nst && q < nst; ++q) issue(q, q);
 
-  float2 acc[TA][TA];
+  float2 acc[TS][TS];
 #pragma unroll
-  for (int i = 0; i < TA; ++i)
+  for (int i = 0; i < TS; ++i)
 #pragma unroll
-    for (int j = 0; j < TA; ++j) acc[i][j] = make_float2(0.f, 0.f);
-
-  if (tid == 0)
-    for (int q = 0; q < kStagesX - 1; ++q) issue(q);
-
-  // rows [I0, I1) of this thread's part, compile-time per branch
-  auto run = [&](auto I0c, auto I1c) {
-    constexpr int I0 = decltype(I0c)::value, I1 = decltype(I1c)::value;
-    int q = 0;
-    for (; q < nst; ++q) {
-      if (tid == 0) issue(q + kStagesX - 1);  // the slot of stage q-1, freed by the sync below
-      const int slot = q % kStagesX;
-      uint32_t ok = 0;
-      for (long long it = 0; it < p.wait_limit && !ok; ++it) {
-        asm volatile(
-            "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-            : "=r"(ok)
-            : "r"(xs_u32(&full[slot])), "r"((uint32_t)((q / kStagesX) & 1))
-            : "memory");
-        if ((it & 1023) == 1023 && s_abort) break;
-      }
-      if (!ok) s_abort = 1;
-      __syncthreads();
-      if (s_abort) break;
-      const unsigned char* st = ring + (size_t)slot * stage_bytes;
-#pragma unroll
-      for (int bi = 0; bi < NB; ++bi) {
-        if (b_lo + q * NB + bi >= b_hi) break;
-        float2 a[TA];
-#pragma unroll
-        for (int i = I0; i < TA; ++i) a[i] = i < S ? ring_value<IN>(st, (bi * S + i) * kXT + lane_ch) : make_float2(0.f, 0.f);
-#pragma unroll
-        for (int i = I0; i < I1; ++i) {
-          const float2 ar = rot_conj(a[i]);
-#pragma unroll
-          for (int j = i; j < TA; ++j)
-            acc[i][j] = j == i ? cmac_auto(acc[i][j], a[i]) : cmac_conj(acc[i][j], a[i], ar, a[j]);
-        }
-      }
-      __syncthreads();
+    for (int j = i; j < TS; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  int slot = 0, turn = 0;
+  uint32_t phase = 0;
+  // lanes beyond the staged channels read the row's first value (their sums are not used)
+  const int lane_off = ((int)threadIdx.x < sh.pitch ? (int)threadIdx.x : 0) * EB;
+  for (int q = 0; q < nst; ++q) {
+    if (q >= 2 && q - 2 + sh.nst < nst && warp == turn && lane == 0) {
+      const int old = ring.reclaim(slot, phase);
+      if (old >= 0) issue(q - 2 + sh.nst, old);
     }
-    if (s_abort) {
-      // let the copies already issued land before the CTA's shared memory
-      // goes away: stage q (whose wait gave up) and the ones issued after it
-      if (tid == 0) {
-        for (int r = q; r < q + kStagesX && r < nst; ++r) {
-          const int slot = r % kStagesX;
-          uint32_t ok = 0;
-          for (long long it = 0; it < kXDrainLimit && !ok; ++it)
-            asm volatile(
-                "{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
-                : "=r"(ok)
-                : "r"(xs_u32(&full[slot])), "r"((uint32_t)((r / kStagesX) & 1))
-                : "memory");
-        }
-        if (p.err) atomicExch(p.err, 1);
-      }
-      return;
+    if (++turn == sh.cg) turn = 0;
+    __syncwarp();
+    if (!ring_wait(&s_full[slot], phase, &s_abort, p.wait_limit)) {
+      s_abort = 1;
+      break;
     }
-    if (k >= p.nchan) return;
-    const int nbl = nbl_of(S);
-#pragma unroll
-    for (int i = I0; i < I1; ++i)
-#pragma unroll
-      for (int j = i; j < TA; ++j)
-        if (i < S && j < S) {
-          float* dst = reinterpret_cast<float*>(p.part + (((size_t)kz * nbl + bl_index(i, j, S)) * p.G + g) *
-                                                             (size_t)p.nchan + k);
-          if (j == i) {
-            atomicAdd(dst, auto_value(acc[i][j]).x);
-          } else {
-            atomicAdd(dst, acc[i][j].x);
-            atomicAdd(dst + 1, acc[i][j].y);
-          }
-        }
-  };
-  constexpr int SPLIT = tri_split(TA, 2, 1);
-  if (part == 0)
-    run(std::integral_constant<int, 0>{}, std::integral_constant<int, SPLIT>{});
-  else
-    run(std::integral_constant<int, SPLIT>{}, std::integral_constant<int, TA>{});
+    const unsigned char* st = data + slot * sh.stage_bytes + lane_off;
+    const int nb = min(sh.nb, b_hi - b_lo - q * sh.nb);
+    for (int bi = 0; bi < nb; ++bi, st += TS * row_bytes) tile_block<TS, IN, true>(acc, st, st, row_bytes);
+    ring.release(slot);
+    if (++slot == sh.nst) {
+      slot = 0;
+      phase ^= 1;
+    }
+  }
+  if (k < p.nchan) {
+    const size_t row = (size_t)p.G * p.nchan;
+    add_tile<TS, true>(acc, p.part + (size_t)kz * nbl_of(TS) * row + (size_t)g * p.nchan + k, row, 0, 0, TS);
+  }
+  __syncthreads();
+  if (s_abort && threadIdx.x == 0) ring.drain(p.err);
 }
 
-static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
-  static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+// More than 12 stations: one CTA takes the tile pairs of group blockIdx.x %
+// groups (the groups of the same 32 channels are neighbours, so that they
+// share L2 lines), stream blockIdx.y and block range blockIdx.z.  A ring stage
+// holds nb blocks of the group's tiles, [tile][block][station][channel], one
+// tensor copy per tile.
+//
+// Bound by the FMA pipe and the register moves of its paired operands: at TS =
+// 8 a warp issues 136 packed FMAs (two cycles each) for 16 shared-memory loads
+// a block.  Twelve pairs a CTA need a station's values from L2 less than half
+// as often as single 8 x 8 pairs, whose L2 traffic bound the step before.
+// Copies of 256-byte rows run at about 13 cycles a row plus 60 a copy, hence
+// several blocks per copy (single blocks reach 3.9 TB/s where the FMAs consume
+// 5.5); 16-byte cp.async copies by the multiplying warps took as much of their
+// time again as the multiplications (2.08 ms for 64 stations x 8 streams x
+// 4096 channels x 128 blocks, 1.58 ms now, 44 TFLOP/s; single 8 x 8 pairs took
+// 3.25 ms).
+template <int TS>
+__global__ void __launch_bounds__(32 * kGroupWarps, 1)
+k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams p, const XShape sh,
+         const __grid_constant__ XGroups groups) {
+  extern __shared__ __align__(128) unsigned char ring_raw[];
+  unsigned char* data = ring_raw + ((128u - (xs_u32(ring_raw) & 127u)) & 127u);
+  __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
+  __shared__ volatile int s_abort, s_issued;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const XGroup& gr = groups.g[blockIdx.x % groups.n];
+  const int k0 = blockIdx.x / groups.n * 32;
+  const int g = blockIdx.y, kz = blockIdx.z, S = p.S;
+  const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
+  const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
+  if (b_hi <= b_lo) return;
+  const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
+  const int row_bytes = sh.pitch * 8, nwarp = gr.nwarp;
+  Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
+  ring.init(nwarp);
+  auto issue = [&](int q, int slot) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xs_u32(&s_full[slot])),
+                 "r"(gr.ntile * sh.nb * TS * row_bytes)
+                 : "memory");
+    for (int i = 0; i < gr.ntile; ++i)
+      asm volatile(
+          "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+          "[%5];" ::"r"(xs_u32(data) + (uint32_t)(slot * sh.stage_bytes + i * sh.tile_bytes)),
+          "l"(reinterpret_cast<uint64_t>(&tmap)), "r"(2 * k0), "r"((int)gr.tile[i] * TS),
+          "r"(g * p.CB + b_lo + q * sh.nb), "r"(xs_u32(&s_full[slot]))
+          : "memory");
+    s_issued = q + 1;
+  };
+  if (threadIdx.x == 0)
+    for (int q = 0; q < sh.nst && q < nst; ++q) issue(q, q);
+
+  // lanes beyond the staged channels read the row's first value (their sums are not used)
+  const int lane_off = (lane < sh.pitch ? lane : 0) * 8;
+  auto run = [&](auto diag, int wa, int wb) {
+    constexpr bool DIAG = decltype(diag)::value;
+    float2 acc[TS][TS];
+#pragma unroll
+    for (int i = 0; i < TS; ++i)
+#pragma unroll
+      for (int j = DIAG ? i : 0; j < TS; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    int slot = 0, turn = 0;
+    uint32_t phase = 0;
+    for (int q = 0; q < nst; ++q) {
+      if (q >= 2 && q - 2 + sh.nst < nst && warp == turn && lane == 0) {
+        const int old = ring.reclaim(slot, phase);
+        if (old >= 0) issue(q - 2 + sh.nst, old);
+      }
+      if (++turn == nwarp) turn = 0;
+      __syncwarp();
+      if (!ring_wait(&s_full[slot], phase, &s_abort, p.wait_limit)) {
+        s_abort = 1;
+        break;
+      }
+      const unsigned char* st = data + slot * sh.stage_bytes + lane_off;
+      const int nb = min(sh.nb, b_hi - b_lo - q * sh.nb);
+      for (int bi = 0; bi < nb; ++bi, st += TS * row_bytes)
+        tile_block<TS, 0, DIAG>(acc, st + wa * sh.tile_bytes, st + wb * sh.tile_bytes, row_bytes);
+      ring.release(slot);
+        if (++slot == sh.nst) {
+        slot = 0;
+        phase ^= 1;
+      }
+    }
+    if (k0 + lane < p.nchan) {
+      const size_t row = (size_t)p.G * p.nchan;
+      add_tile<TS, DIAG>(acc, p.part + (size_t)kz * nbl_of(S) * row + (size_t)g * p.nchan + k0 + lane, row,
+                         gr.tile[wa] * TS, gr.tile[wb] * TS, S);
+    }
+  };
+  if (warp < nwarp) {  // a CTA with fewer pairs than the largest one has warps without work
+    const int wa = gr.wa[warp], wb = gr.wb[warp];
+    if (wa == wb) run(std::true_type{}, wa, wb);
+    else run(std::false_type{}, wa, wb);
+  }
+  __syncthreads();
+  if (s_abort && threadIdx.x == 0) ring.drain(p.err);
+}
+
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+  static const PFN_cuTensorMapEncodeTiled_v12000 fn = [] {
     void* ptr = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &ptr, 12000, cudaEnableDefault, &q) == cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
-    else
-      cudaGetLastError();
-  }
+      return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(ptr);
+    cudaGetLastError();
+    return (PFN_cuTensorMapEncodeTiled_v12000) nullptr;
+  }();
   return fn;
 }
 
-// The tensor map views the spectra as rows (stream, block, station) of 2 nchan
-// scalars (Re, Im interleaved): FP32, FP16 or single bytes (E4M3 pairs); a
-// stage is 2 x 128 scalars (128 channels, 256..1024 bytes, a multiple of 16)
-// by NB * S rows (NB blocks per stage), from x = 2 k0 (a multiple of 256 scalars).
-template <int TA, int IN>
-static cudaError_t launch_tma_in(const XParams& p_in, cudaStream_t s, bool* used) {
-  *used = false;
-  XParams p = p_in;
-  p.wait_limit = wait_limit();
+// Stations per tile above kOneTile: the size whose tile pairs cost least per
+// block, counting packed FMAs (an autocorrelation takes one, a baseline two,
+// a station one) and each shared-memory load as two of them.  Small tiles
+// waste less on stations beyond S, large ones load less: 20 stations go as
+// 7 + 7 + 6, not 8 + 8 + 4 or 4 x 5.
+int tile_size(int S) {
+  if (S > 64) return 8;
+  int best = 8;
+  long cost = 0;
+  for (int ts = 8; ts >= 5; --ts) {
+    const long nt = (S + ts - 1) / ts;
+    const long c = nt * (ts * ts + 3 * ts) + nt * (nt - 1) / 2 * (2 * ts * ts + 5 * ts);
+    if (ts == 8 || c < cost) {
+      best = ts;
+      cost = c;
+    }
+  }
+  return best;
+}
+
+// Tile pairs in CTAs: in blocks of 4 x 4 tiles, so that consecutive pairs
+// share tiles (64 stations: 36 pairs in three CTAs that stage 6, 8 and 5 of
+// the 8 tiles).  A CTA of 12 warps fills an SM; with fewer pairs, CTAs of a
+// size that several of them nearly fill one.
+XGroups make_groups(int nt) {
+  struct Pair { int a, b; };
+  Pair pairs[kMaxTiles * (kMaxTiles + 1) / 2];
+  int n = 0;
+  for (int I = 0; I < nt; I += 4)
+    for (int J = I; J < nt; J += 4)
+      for (int a = I; a < std::min(I + 4, nt); ++a)
+        for (int b = std::max(a, J); b < std::min(J + 4, nt); ++b) pairs[n++] = {a, b};
+  const int least = (n + kGroupWarps - 1) / kGroupWarps;
+  int size = kGroupWarps;
+  double best = 0.0;
+  for (int ng = least; ng < least + 3; ++ng) {
+    const int sz = (n + ng - 1) / ng;
+    const double warps = (double)(kGroupWarps / sz) * n / ng;
+    if (warps > best) {
+      best = warps;
+      size = sz;
+    }
+  }
+  XGroups out;
+  memset(&out, 0, sizeof(out));
+  for (int q = 0; q < n;) {
+    XGroup& x = out.g[out.n++];
+    for (; q < n && x.nwarp < size; ++q) {
+      int at[2];
+      const int t[2] = {pairs[q].a, pairs[q].b};
+      int have = x.ntile;
+      for (int e = 0; e < 2; ++e) {
+        int i = 0;
+        while (i < have && x.tile[i] != t[e]) ++i;
+        if (i == have) {
+          if (have == kGroupTiles) { i = -1; }
+          else x.tile[have++] = (uint8_t)t[e];
+        }
+        at[e] = i;
+        if (i < 0) break;
+      }
+      if (at[0] < 0 || at[1] < 0) break;  // no room for its tiles: the next CTA's first pair
+      x.ntile = (uint8_t)have;
+      x.wa[x.nwarp] = (uint8_t)at[0];
+      x.wb[x.nwarp++] = (uint8_t)at[1];
+    }
+    // pairs inside a tile have half the work: first, so that they go to
+    // different schedulers (warp % 4)
+    for (int w = 0, d = 0; w < x.nwarp; ++w)
+      if (x.wa[w] == x.wb[w]) {
+        std::swap(x.wa[w], x.wa[d]);
+        std::swap(x.wb[w], x.wb[d++]);
+      }
+  }
+  return out;
+}
+
+struct XPlan {
+  int ts, cg, pitch, ngroup, warps, ctas_per_sm;
+  int tiles;  // staged per CTA, at most
+};
+
+XPlan plan_for(int S, int nchan, XGroups* groups) {
+  XPlan x;
+  if (S <= kOneTile) {
+    x.ts = S;
+    x.cg = nchan >= 128 ? 4 : (nchan + 31) / 32;
+    x.pitch = std::min(nchan, 32 * x.cg);
+    x.ngroup = x.tiles = 1;
+    x.warps = x.cg;
+    x.ctas_per_sm = one_tile_ctas(S);
+    return x;
+  }
+  x.ts = tile_size(S);
+  x.cg = 1;
+  x.pitch = std::min(nchan, 32);
+  const XGroups g = make_groups((S + x.ts - 1) / x.ts);
+  x.ngroup = g.n;
+  x.warps = x.tiles = 0;
+  for (int i = 0; i < g.n; ++i) {
+    x.warps = std::max(x.warps, (int)g.g[i].nwarp);
+    x.tiles = std::max(x.tiles, (int)g.g[i].ntile);
+  }
+  x.ctas_per_sm = kGroupWarps / x.warps;
+  if (groups) *groups = g;
+  return x;
+}
+
+// The ring of a launch: at least four stages (more if a block is small) of up
+// to `most` blocks in a CTA's share of 216 KB of shared memory, and the tensor
+// map: the spectra as [stream x block][station][2 nchan scalars], FP32, FP16
+// or single bytes (E4M3 pairs); a copy takes 2 pitch scalars (a multiple of 16
+// bytes, from a multiple of 64 scalars) x TS stations (zeros beyond S) x nb
+// blocks.
+template <int TS, int IN>
+cudaError_t ring_shape(const XParams& p, const XPlan& x, int most, XShape* sh, CUtensorMap* tm, size_t* smem) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
-  constexpr int EB = SpecElem<IN>::bytes;
-  constexpr int NB = SpecElem<IN>::nb;
-  if (!enc || p.nchan < kXT || p.nchan % kXT || NB * p.S > 256) return cudaSuccess;
-  CUtensorMap tm;
-  cuuint64_t dims[2] = {(cuuint64_t)2 * p.nchan, (cuuint64_t)p.G * p.CB * p.S};
-  cuuint64_t strides[1] = {(cuuint64_t)p.nchan * EB};
-  cuuint32_t box[2] = {(cuuint32_t)(2 * kXT), (cuuint32_t)(NB * p.S)};
-  cuuint32_t estr[2] = {1, 1};
+  if (!enc) return cudaErrorNotSupported;
+  constexpr int EB = spec_bytes(IN);
+  const int block_bytes = TS * x.pitch * EB, budget = 216 * 1024 / x.ctas_per_sm;
+  sh->cg = x.cg;
+  sh->pitch = x.pitch;
+  sh->nb = std::max(1, std::min({most, p.CB / std::max(1, p.KZ), budget / 4 / (x.tiles * block_bytes)}));
+  sh->tile_bytes = (sh->nb * block_bytes + 127) & ~127;
+  sh->stage_bytes = x.tiles * sh->tile_bytes;
+  sh->nst = std::min(kMaxStages, budget / sh->stage_bytes);
+  *smem = 128 + (size_t)sh->nst * sh->stage_bytes;
+  cuuint64_t dims[3] = {(cuuint64_t)2 * p.nchan, (cuuint64_t)p.S, (cuuint64_t)p.G * p.CB};
+  cuuint64_t strides[2] = {(cuuint64_t)p.nchan * EB, (cuuint64_t)p.S * p.nchan * EB};
+  cuuint32_t box[3] = {(cuuint32_t)(2 * x.pitch), (cuuint32_t)TS, (cuuint32_t)sh->nb};
+  cuuint32_t estr[3] = {1, 1, 1};
   const CUtensorMapDataType dt =
       IN == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : (IN == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8);
-  if (enc(&tm, dt, 2, const_cast<float2*>(p.spec), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaSuccess;  // FP32: fall back to the cp.async ring
-  const size_t smem = 1024 + (size_t)kStagesX * NB * p.S * kXT * EB;
-  cudaError_t e = cudaFuncSetAttribute(k_xmac_tma<TA, IN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return enc(tm, dt, 3, const_cast<float2*>(p.spec), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS
+             ? cudaSuccess
+             : cudaErrorInvalidValue;
+}
+
+template <int TS, int IN>
+cudaError_t launch_one_in(const XParams& p_in, const XPlan& x, cudaStream_t s) {
+  XParams p = p_in;
+  p.wait_limit = wait_limit();
+  XShape sh;
+  CUtensorMap tm;
+  size_t smem = 0;
+  cudaError_t e = ring_shape<TS, IN>(p, x, 16, &sh, &tm, &smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_xmac<TS, IN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  dim3 grid((p.nchan + kXT - 1) / kXT, p.G, p.KZ);
-  k_xmac_tma<TA, IN><<<grid, kXThreadsT, smem, s>>>(tm, p);
-  *used = true;
+  k_xmac<TS, IN><<<dim3((p.nchan + 32 * x.cg - 1) / (32 * x.cg), p.G, p.KZ), 32 * x.cg, smem, s>>>(tm, p, sh);
   return cudaGetLastError();
 }
 
-template <int TA>
-static cudaError_t launch_tma(const XParams& p, cudaStream_t s, bool* used) {
-  if (p.in_kind == 1) return launch_tma_in<TA, 1>(p, s, used);
-  if (p.in_kind == 2) return launch_tma_in<TA, 2>(p, s, used);
-  return launch_tma_in<TA, 0>(p, s, used);
+template <int TS>
+cudaError_t launch_one(const XParams& p, const XPlan& x, cudaStream_t s) {
+  if (p.in_kind == 1) return launch_one_in<TS, 1>(p, x, s);
+  if (p.in_kind == 2) return launch_one_in<TS, 2>(p, x, s);
+  return launch_one_in<TS, 0>(p, x, s);
 }
 
-static int tile_for(int S) {
-  if (S <= 2) return 2;
-  if (S <= 4) return 4;
-  if (S <= 6) return 6;
-  if (S <= 8) return 8;
-  if (S <= 10) return 10;
-  if (S <= 12) return 12;
-  return 8;
+template <int TS>
+cudaError_t launch_pairs(const XParams& p_in, const XPlan& x, const XGroups& groups, cudaStream_t s) {
+  XParams p = p_in;
+  p.wait_limit = wait_limit();
+  XShape sh;
+  CUtensorMap tm;
+  size_t smem = 0;
+  cudaError_t e = ring_shape<TS, 0>(p, x, 4, &sh, &tm, &smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_xpairs<TS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_xpairs<TS><<<dim3(x.ngroup * ((p.nchan + 31) / 32), p.G, p.KZ), 32 * x.warps, smem, s>>>(tm, p, sh, groups);
+  return cudaGetLastError();
 }
 
+}  // namespace
+
+// Block ranges per chunk.  At least one per 256 blocks (the length of an FP32
+// register sum); above that the number whose CTAs fill whole waves of the
+// SMs, weighed against each CTA's start and end (worth about 12 blocks) and
+// the partial sums it adds to memory (read and written, against the spectra
+// read).
 int xstage_kz(int CB, int S, int G, int nchan) {
-  const int TA = tile_for(S);
-  const int nt = (S + TA - 1) / TA;
-  const long ctas = (long)((nchan + kXT - 1) / kXT) * G * (nt * (nt + 1) / 2);
-  // about three waves of two CTAs per SM
-  int kz = (int)((3L * 2 * 152 + ctas - 1) / ctas);
-  const int by256 = (CB + 255) / 256;            // each partial sums <= 256 blocks
-  if (kz < by256) kz = by256;
-  if (kz > CB) kz = CB;
-  if (kz < 1) kz = 1;
-  return kz;
-}
-
-template <int TA>
-static cudaError_t launch_ring(const XParams& p, cudaStream_t s) {
-  bool used = false;
-  cudaError_t te = launch_tma<TA>(p, s, &used);
-  if (te != cudaSuccess || used) return te;
-  if (p.in_kind != 0) return cudaErrorNotSupported;  // FP16 / E4M3 spectra: the TMA ring only
-  const size_t smem = (size_t)kStagesX * kNB * p.S * kXT * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_xmac_ring<TA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((p.nchan + kXT - 1) / kXT, p.G, p.KZ);
-  k_xmac_ring<TA><<<grid, kXT, smem, s>>>(p);
-  return cudaGetLastError();
-}
-
-template <int TA>
-static cudaError_t launch_TA(const XParams& p, cudaStream_t s) {
-  const int nt = (p.S + TA - 1) / TA;
-  const int ntiles = (p.nchan + kXT - 1) / kXT;
-  const size_t smem1 = (size_t)kStagesT * TA * kXT * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_xmac<TA, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-  if (e != cudaSuccess) return e;
-  k_xmac<TA, true><<<dim3(nt * ntiles, p.G, p.KZ), 2 * kXT, smem1, s>>>(p, nt);
-  if ((e = cudaGetLastError()) != cudaSuccess || nt == 1) return e;
-  if constexpr (TA == 8) {  // only the 8-station tiling has off-diagonal tiles
-    const size_t smem2 = 2 * smem1;
-    e = cudaFuncSetAttribute(k_xmac<TA, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2);
-    if (e != cudaSuccess) return e;
-    k_xmac<TA, false><<<dim3(nt * (nt - 1) / 2 * ntiles, p.G, p.KZ), 2 * kXT, smem2, s>>>(p, nt);
-    return cudaGetLastError();
+  const XPlan x = plan_for(S, nchan, nullptr);
+  const int64_t base = (int64_t)x.ngroup * ((nchan + 32 * x.cg - 1) / (32 * x.cg)) * G;
+  const int64_t slots = (int64_t)152 * x.ctas_per_sm;
+  const int least = std::max(1, (CB + 255) / 256);
+  const int most = (int)std::min<int64_t>(CB, std::max<int64_t>(least, 3 * slots / base + 1));
+  int best = least;
+  double score = 0.0;
+  for (int kz = least; kz <= most; ++kz) {
+    const int64_t ctas = base * kz, waves = (ctas + slots - 1) / slots;
+    const double nb = (double)CB / kz;
+    const double v = (double)ctas / (double)(waves * slots) * nb / (nb + 12.0) / (1.0 + (S + 1.0) / nb);
+    if (v > score) {
+      score = v;
+      best = kz;
+    }
   }
-  return cudaErrorInvalidValue;
+  return std::min(best, std::max(1, CB));
 }
 
 bool xstage_reduced_supported(int S, int nchan) {
-  return S >= 1 && S <= 12 && SpecElem<2>::nb * S <= 256 && nchan >= kXT && nchan % kXT == 0 &&
-         tensor_map_encoder() != nullptr;
+  return S >= 1 && S <= kOneTile && nchan >= 128 && nchan % 128 == 0 && tensor_map_encoder() != nullptr;
 }
 
 cudaError_t launch_xstage(const XParams& p, cudaStream_t s) {
   if (p.CB <= 0) return cudaSuccess;
   if (p.in_kind != 0 && !xstage_reduced_supported(p.S, p.nchan)) return cudaErrorNotSupported;
-  switch (tile_for(p.S)) {
-    case 2: return launch_ring<2>(p, s);
-    case 4: return launch_ring<4>(p, s);
-    case 6: return launch_ring<6>(p, s);
-    case 8: return p.S <= 8 ? launch_ring<8>(p, s) : launch_TA<8>(p, s);
-    case 10: return launch_ring<10>(p, s);
-    case 12: return launch_ring<12>(p, s);
-    default: return cudaErrorInvalidValue;
+  if (p.S > kMaxXStations) return cudaErrorInvalidValue;
+  XGroups groups;
+  const XPlan x = plan_for(p.S, p.nchan, &groups);
+  if (p.S <= kOneTile) {
+    switch (x.ts) {
+      case 1: return launch_one<1>(p, x, s);
+      case 2: return launch_one<2>(p, x, s);
+      case 3: return launch_one<3>(p, x, s);
+      case 4: return launch_one<4>(p, x, s);
+      case 5: return launch_one<5>(p, x, s);
+      case 6: return launch_one<6>(p, x, s);
+      case 7: return launch_one<7>(p, x, s);
+      case 8: return launch_one<8>(p, x, s);
+      case 9: return launch_one<9>(p, x, s);
+      case 10: return launch_one<10>(p, x, s);
+      case 11: return launch_one<11>(p, x, s);
+      case 12: return launch_one<12>(p, x, s);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  switch (x.ts) {
+    case 5: return launch_pairs<5>(p, x, groups, s);
+    case 6: return launch_pairs<6>(p, x, groups, s);
+    case 7: return launch_pairs<7>(p, x, groups, s);
+    default: return launch_pairs<8>(p, x, groups, s);
   }
 }
 
