@@ -146,6 +146,7 @@ cudaError_t launch_fstage(const FParams& p, cudaStream_t s);
 bool fstage_pre_supported(int nchan);
 cudaError_t launch_fstage_pre(const FParams& p, cudaStream_t s);
 cudaError_t fstage_pre_init_constants();
+cudaError_t fringe_init_constants();
 int xstage_kz(int CB, int S, int G, int nchan);
 cudaError_t launch_xstage(const XParams& p, cudaStream_t s);
 cudaError_t launch_weights(const FinParams& p, cudaStream_t s);

@@ -5,97 +5,259 @@
 // zero-padded two-dimensional inverse DFT, unnormalised,
 //     M[r][l] = sum_t sum_k V[t][k] exp(+2 pi i (k l / Nd + t r / Nr)),
 // and the peak is the largest |M|, the smaller flat index r * Nd + l on ties.
-// Two passes of a shared-memory radix-2 complex FFT (one CTA per transform):
-// over channels for every sub-integration (written transposed, lag-major),
-// then over sub-integrations for every lag; then one reduction for the peak.
+// Two passes of k_cfft_inv: over channels for every sub-integration, then over
+// sub-integrations for every lag, whose last pass also finds the peak.
 #include "../../include/corr.h"
-#include "corr_internal.cuh"
+#include "k_fstage_impl.cuh"
 
+#include <atomic>
 #include <math.h>
 #include <stdint.h>
 #include <string.h>
 
 namespace corr {
 
+cudaError_t fringe_init_constants() { return init_w32(); }
+
 namespace {
 
-constexpr int kFftThreads = 512;
 constexpr int kMaxFft = 16384;
 
-__device__ __forceinline__ int bitrev(int x, int bits) { return (int)(__brev((unsigned)x) >> (32 - bits)); }
+// The peak of one search: `best` orders by amplitude, then by smaller index.
+struct PeakSlot {
+  unsigned long long best;
+  unsigned int done;  // finished CTAs of the second pass
+  float2 value;       // the map at the peak, written by the last of them
+};
 
-// One inverse transform of length n (a power of two) per CTA: row `row` of
-// `in` (in_len values, the rest zero) -> out[row * orow + i * ocol], i < n.
-// Iterative radix-2 decimation in time on a bit-reversed copy in shared
-// memory; the twiddles exp(+2 pi i j / n), j < n/2, come from sincospif.
-__global__ void __launch_bounds__(kFftThreads) k_cfft_inv(const float2* __restrict__ in, int in_len, int64_t in_ld,
-                                                          float2* __restrict__ out, int n, int logn, int64_t orow,
-                                                          int64_t ocol) {
-  extern __shared__ __align__(16) float2 sm[];
-  float2* s = sm;          // [n]
-  float2* tw = sm + n;     // [n / 2]
-  const int row = blockIdx.x;
-  const float2* src = in + (int64_t)row * in_ld;
-  for (int j = threadIdx.x; j < n / 2; j += blockDim.x) {
+// A search holds one slot from its first launch until it has read the peak
+// back (the call waits for that), so concurrent searches on other threads and
+// streams have slots of their own.
+constexpr int kPeakSlots = 64;
+__device__ PeakSlot g_peak_slots[kPeakSlots];
+std::atomic<unsigned long long> g_peak_taken{0};
+
+// Radices of a transform of n = R0 R1 R2 points.  A thread holds 32 points
+// (n if fewer) in every pass.
+template <int n> struct Radices {
+  static constexpr int R0 = n <= 32 ? n : n == 64 ? 8 : (n == 512 || n == 1024 || n == 16384) ? 32 : 16;
+  static constexpr int R1 = n <= 32 ? 1 : (n == 64 || n == 128) ? 8 : (n == 1024 || n == 16384) ? 32 : 16;
+  static constexpr int R2 = n / R0 / R1;  // 1, 8, 16 or 32
+  static constexpr int T = n <= 32 ? 1 : n / 32;
+  static_assert(R0 * R1 * R2 == n, "radices");
+};
+
+// Transforms per CTA: rows (consecutive in memory) fill about 256 threads;
+// of columns up to 16 (one 128-byte line a row of the map) as long as their
+// points fit 64 KB of shared memory and 256 threads, more for short ones.
+template <int n, bool COLS> struct Batch {
+  static constexpr int T = Radices<n>::T;
+  static constexpr int C = T >= 256 ? 1 : COLS ? (n <= 64 ? 128 / T : n <= 256 ? 32 : 8192 / n) : 256 / T > 64 ? 64 : 256 / T;
+};
+
+// Position of point i of transform c in shared memory: columns side by side
+// (the threads of a warp run over columns), rows one after another with a
+// padding element after every R0 points.
+template <int n, bool COLS>
+__device__ __forceinline__ int at(int i, int c) {
+  if constexpr (COLS) return i * Batch<n, COLS>::C + c;
+  else return c * (n + n / Radices<n>::R0 + 1) + padp<Radices<n>::R0>(i);
+}
+
+// v[r] *= W_{NS R}^{-k r}: the powers k 2^i from sincospif, whose argument is
+// exact, and the rest as their products.  The transforms work on swapped
+// (imaginary, real) values, which turns the forward butterflies of dft_reg
+// into inverse ones, so the twiddles here are the forward ones.
+template <int R, int NS>
+__device__ __forceinline__ void cfft_twiddle(float2 (&v)[R], int k) {
+  constexpr int LOGR = ilog2c(R);
+  float2 wp[LOGR];
+#pragma unroll
+  for (int i = 0; i < LOGR; ++i) {
     float sn, cs;
-    sincospif(2.0f * (float)j / (float)n, &sn, &cs);
-    tw[j] = make_float2(cs, sn);
+    sincospif(-2.0f * (float)(k << i) / (float)(NS * R), &sn, &cs);
+    wp[i] = make_float2(cs, sn);
   }
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const int j = bitrev(i, logn);
-    s[i] = j < in_len ? src[j] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  for (int half = 1; half < n; half <<= 1) {
-    const int step = n / (2 * half);  // twiddle index stride for this stage
-    for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
-      const int p = b & (half - 1);
-      const int i0 = ((b - p) << 1) + p;
-      const int i1 = i0 + half;
-      const float2 w = tw[p * step];
-      const float2 u = s[i0], x = s[i1];
-      const float2 v = make_float2(x.x * w.x - x.y * w.y, x.x * w.y + x.y * w.x);
-      s[i0] = make_float2(u.x + v.x, u.y + v.y);
-      s[i1] = make_float2(u.x - v.x, u.y - v.y);
+  twiddle_products<R, LOGR>(v, wp);
+}
+
+// A middle or last pass: R points a butterfly from shared memory; the middle
+// one back to it, the last one to `store`.
+template <int n, int R, int NS, bool COLS, typename Store>
+__device__ __forceinline__ void cfft_pass(float2* buf, int t, int c, Store store) {
+  constexpr int T = Radices<n>::T, PER = n / R / T;
+  constexpr bool last = NS * R == n;
+  float2 v[PER][R];
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[u][r] = buf[at<n, COLS>(t + u * T + r * (n / R), c)];
+  if constexpr (!last) __syncthreads();
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int j = t + u * T, k = j & (NS - 1);
+    cfft_twiddle<R, NS>(v[u], k);
+    dft_reg<R>(v[u]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      if constexpr (last) store(k + r * NS, v[u][r]);
+      else buf[at<n, COLS>((j / NS) * NS * R + k + r * NS, c)] = v[u][r];
     }
-    __syncthreads();
   }
-  float2* dst = out + (int64_t)row * orow;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[(int64_t)i * ocol] = s[i];
+  if constexpr (!last) __syncthreads();
 }
 
-// Largest amplitude with the smallest flat index on ties: one 64-bit key per
-// element, amplitude bits (non-negative floats order like their bit
-// patterns) above the complement of the index, reduced with atomicMax.
-__global__ void __launch_bounds__(256) k_fringe_peak(const float2* __restrict__ map, int64_t count,
-                                                     unsigned long long* __restrict__ best) {
+// Amplitude bits (non-negative floats order like their bit patterns) above
+// the complement of the flat index: the largest key is the largest amplitude
+// with the smallest index.
+__device__ __forceinline__ unsigned long long peak_key(float2 v, uint32_t e) {
+  const float a = sqrtf(v.x * v.x + v.y * v.y);
+  return ((unsigned long long)__float_as_uint(a) << 32) | (unsigned long long)(0xFFFFFFFFu - e);
+}
+
+// Inverse transforms of n points, C per CTA: transform q (a row, or with COLS
+// a column) has point i at in[q * in_q + i * in_i] for i < in_len, zero above,
+// and writes point i to out[q * out_q + i * out_i].
+//
+// Bound by the map's one write and by latency (a few waves of CTAs at most).
+// The points stay in registers (radix 8..32 passes) and cross shared memory
+// once or twice; the first pass reads global memory, the last one writes it.
+// The rows' results lie in the map's own first in_len rows: a CTA of the
+// second pass reads its columns before it writes them, whole 128-byte lines
+// for transforms of up to 512 points, so the search needs no work space.
+// 256 x 1024 values into 512 x 8192 bins: 12.9 + 21.3 us (radix-2 passes in
+// shared memory, a transposed write of the lags and a pass of its own for the
+// peak took 66.6 + 70.7 + 11.0 us).
+template <int n, bool COLS, bool PEAK>
+__global__ void __launch_bounds__(Radices<n>::T * Batch<n, COLS>::C)
+k_cfft_inv(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out, int64_t out_q, int64_t out_i,
+           int count, PeakSlot* slot) {
+  using P = Radices<n>;
+  constexpr int T = P::T, C = Batch<n, COLS>::C, PER = n / P::R0 / T;
+  extern __shared__ __align__(16) float2 cfft_buf[];
+  const int c = COLS ? threadIdx.x % C : threadIdx.x / T;
+  const int t = COLS ? threadIdx.x / C : threadIdx.x % T;
+  const int q = blockIdx.x * C + c;
+  const bool mine = q < count;
+  if (!PEAK && blockIdx.x == 0 && threadIdx.x == 0) {  // the next pass finds the slot cleared
+    slot->best = 0ull;
+    slot->done = 0u;
+  }
   unsigned long long key = 0ull;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
-    const float2 v = map[e];
-    const float a = sqrtf(v.x * v.x + v.y * v.y);
-    const unsigned long long k =
-        ((unsigned long long)__float_as_uint(a) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)e);
-    key = k > key ? k : key;
+  auto store = [&](int i, float2 v) {
+    if (!mine) return;
+    v = swp(v);
+    out[q * out_q + i * out_i] = v;
+    if constexpr (PEAK) {
+      const unsigned long long k = peak_key(v, (uint32_t)(q * out_q + i * out_i));
+      key = k > key ? k : key;
+    }
+  };
+  float2 v[PER][P::R0];
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+#pragma unroll
+    for (int r = 0; r < P::R0; ++r) {
+      const int i = t + u * T + r * (n / P::R0);
+      v[u][r] = mine && i < in_len ? swp(in[q * in_q + i * in_i]) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    dft_reg<P::R0>(v[u]);
+#pragma unroll
+    for (int r = 0; r < P::R0; ++r) {
+      if constexpr (P::R1 == 1) store(r, v[u][r]);
+      else cfft_buf[at<n, COLS>((t + u * T) * P::R0 + r, c)] = v[u][r];
+    }
   }
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long other = __shfl_down_sync(0xffffffffu, key, o);
-    key = other > key ? other : key;
+  if constexpr (P::R1 > 1) {
+    __syncthreads();
+    cfft_pass<n, P::R1, P::R0, COLS>(cfft_buf, t, c, store);
+    if constexpr (P::R2 > 1) cfft_pass<n, P::R2, P::R0 * P::R1, COLS>(cfft_buf, t, c, store);
   }
-  __shared__ unsigned long long ws[8];
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = key;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) key = ws[w] > key ? ws[w] : key;
-    atomicMax(best, key);
+  if constexpr (PEAK) {
+    __threadfence();  // the map's values, for the CTA that reads the peak's
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long other = __shfl_down_sync(0xffffffffu, key, o);
+      key = other > key ? other : key;
+    }
+    __shared__ unsigned long long ws[32];
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = key;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) key = ws[w] > key ? ws[w] : key;
+      atomicMax(&slot->best, key);
+      __threadfence();
+      if (atomicAdd(&slot->done, 1u) == gridDim.x - 1) {
+        __threadfence();
+        const unsigned long long best = atomicMax(&slot->best, 0ull);
+        slot->value = __ldcg(out + (0xFFFFFFFFu - (uint32_t)best));
+      }
+    }
   }
 }
 
-int ilog2_exact(int n) {
-  if (n < 2 || (n & (n - 1))) return -1;
-  int l = 0;
-  while ((1 << l) < n) ++l;
-  return l;
+template <int n, bool COLS, bool PEAK>
+cudaError_t launch_cfft_n(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out, int64_t out_q,
+                          int64_t out_i, int count, PeakSlot* slot, cudaStream_t st) {
+  constexpr int C = Batch<n, COLS>::C;
+  constexpr size_t smem = Radices<n>::R1 == 1 ? 0
+                          : sizeof(float2) * (COLS ? (size_t)n * C : (size_t)C * (n + n / Radices<n>::R0 + 1));
+  cudaError_t e = cudaFuncSetAttribute(k_cfft_inv<n, COLS, PEAK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k_cfft_inv<n, COLS, PEAK><<<(count + C - 1) / C, Radices<n>::T * C, smem, st>>>(in, in_len, in_q, in_i, out, out_q,
+                                                                                 out_i, count, slot);
+  return cudaGetLastError();
 }
+
+template <bool COLS, bool PEAK, typename... A>
+cudaError_t launch_cfft(int n, A... a) {
+  switch (n) {
+    case 2: return launch_cfft_n<2, COLS, PEAK>(a...);
+    case 4: return launch_cfft_n<4, COLS, PEAK>(a...);
+    case 8: return launch_cfft_n<8, COLS, PEAK>(a...);
+    case 16: return launch_cfft_n<16, COLS, PEAK>(a...);
+    case 32: return launch_cfft_n<32, COLS, PEAK>(a...);
+    case 64: return launch_cfft_n<64, COLS, PEAK>(a...);
+    case 128: return launch_cfft_n<128, COLS, PEAK>(a...);
+    case 256: return launch_cfft_n<256, COLS, PEAK>(a...);
+    case 512: return launch_cfft_n<512, COLS, PEAK>(a...);
+    case 1024: return launch_cfft_n<1024, COLS, PEAK>(a...);
+    case 2048: return launch_cfft_n<2048, COLS, PEAK>(a...);
+    case 4096: return launch_cfft_n<4096, COLS, PEAK>(a...);
+    case 8192: return launch_cfft_n<8192, COLS, PEAK>(a...);
+    case 16384: return launch_cfft_n<16384, COLS, PEAK>(a...);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+bool is_fft_length(int n) { return n >= 2 && n <= kMaxFft && (n & (n - 1)) == 0; }
+
+// A slot for one search, given back when it goes out of scope; slots beyond
+// the static ones come from the stream's memory pool.
+struct PeakLease {
+  PeakSlot* dev = nullptr;
+  int index = -1;
+  cudaStream_t st;
+  explicit PeakLease(cudaStream_t s) : st(s) {
+    unsigned long long taken = g_peak_taken.load();
+    while (~taken) {
+      const int i = __builtin_ctzll(~taken);
+      if (!g_peak_taken.compare_exchange_weak(taken, taken | (1ull << i))) continue;
+      index = i;
+      void* base = nullptr;
+      if (cudaGetSymbolAddress(&base, g_peak_slots) == cudaSuccess) dev = reinterpret_cast<PeakSlot*>(base) + i;
+      return;
+    }
+    void* p = nullptr;
+    if (cudaMallocAsync(&p, sizeof(PeakSlot), st) == cudaSuccess) dev = reinterpret_cast<PeakSlot*>(p);
+  }
+  ~PeakLease() {
+    if (index >= 0) g_peak_taken.fetch_and(~(1ull << index));
+    else if (dev) cudaFreeAsync(dev, st);
+  }
+  PeakLease(const PeakLease&) = delete;
+};
 
 }  // namespace
 
@@ -107,57 +269,42 @@ extern "C" int corr_fringe_search(const float* dev_vis, int nsub, int nchan, int
                                   float* dev_map, int* peak_rate, int* peak_lag, float* peak_amp,
                                   float* peak_value, void* cuda_stream) {
   if (!dev_vis || !dev_map || nsub < 1 || nchan < 1) return CORR_EINVAL;
-  const int lr = ilog2_exact(pad_rate), ld = ilog2_exact(pad_delay);
-  if (lr < 0 || ld < 0 || pad_rate < nsub || pad_delay < nchan || pad_rate > kMaxFft || pad_delay > kMaxFft ||
+  if (!is_fft_length(pad_rate) || !is_fft_length(pad_delay) || pad_rate < nsub || pad_delay < nchan ||
       (int64_t)pad_rate * pad_delay > ((int64_t)1 << 26))
     return CORR_EINVAL;
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const float2* V = reinterpret_cast<const float2*>(dev_vis);
   float2* M = reinterpret_cast<float2*>(dev_map);
-  // scratch: the lag transforms, lag-major [pad_delay][nsub], plus the peak key
-  const size_t scratch = sizeof(float2) * (size_t)pad_delay * nsub + 256;
+  const int64_t count = (int64_t)pad_rate * pad_delay;
+  cudaError_t e = fstage_ensure_constants();
+  PeakLease lease(st);
+  // the lag transforms [nsub][pad_delay]: the map's first rows, unless the
+  // visibilities themselves lie in the map
+  float2* X1 = M;
   void* buf = nullptr;
-  if (cudaMallocAsync(&buf, scratch, st) != cudaSuccess) {
+  const uintptr_t v0 = (uintptr_t)V, v1 = v0 + sizeof(float2) * (size_t)nsub * nchan, m0 = (uintptr_t)M,
+                  m1 = m0 + sizeof(float2) * (size_t)count;
+  if (!lease.dev || (v0 < m1 && m0 < v1 &&
+                     cudaMallocAsync(&buf, sizeof(float2) * (size_t)pad_delay * nsub, st) != cudaSuccess)) {
     cudaGetLastError();
     return CORR_ENOMEM;
   }
-  float2* X1 = reinterpret_cast<float2*>(buf);
-  unsigned long long* best =
-      reinterpret_cast<unsigned long long*>(reinterpret_cast<char*>(buf) + sizeof(float2) * (size_t)pad_delay * nsub);
-  cudaError_t e = cudaSuccess;
-  const int maxn = pad_rate > pad_delay ? pad_rate : pad_delay;
-  const size_t smem_max = sizeof(float2) * ((size_t)maxn + maxn / 2);
-  e = cudaFuncSetAttribute(k_cfft_inv, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-  // over channels: row t of V -> X1[l][t]
-  if (e == cudaSuccess) {
-    const int thr = pad_delay / 2 < kFftThreads ? (pad_delay / 2 > 32 ? pad_delay / 2 : 32) : kFftThreads;
-    k_cfft_inv<<<nsub, thr, sizeof(float2) * ((size_t)pad_delay + pad_delay / 2), st>>>(V, nchan, nchan, X1,
-                                                                                        pad_delay, ld, 1, nsub);
-    e = cudaGetLastError();
-  }
-  // over sub-integrations: row l of X1 -> M[r][l]
-  if (e == cudaSuccess) {
-    const int thr = pad_rate / 2 < kFftThreads ? (pad_rate / 2 > 32 ? pad_rate / 2 : 32) : kFftThreads;
-    k_cfft_inv<<<pad_delay, thr, sizeof(float2) * ((size_t)pad_rate + pad_rate / 2), st>>>(X1, nsub, nsub, M,
-                                                                                          pad_rate, lr, 1, pad_delay);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemsetAsync(best, 0, sizeof(unsigned long long), st);
-  const int64_t count = (int64_t)pad_rate * pad_delay;
-  if (e == cudaSuccess) {
-    int blocks = (int)((count + 255) / 256);
-    if (blocks > 152 * 8) blocks = 152 * 8;
-    k_fringe_peak<<<blocks, 256, 0, st>>>(M, count, best);
-    e = cudaGetLastError();
-  }
-  unsigned long long key = 0ull;
-  float2 pv = make_float2(0.f, 0.f);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&key, best, sizeof(key), cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  const int64_t idx = (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
+  if (buf) X1 = reinterpret_cast<float2*>(buf);
+  // over channels: row t of V -> X1[t][l]; over sub-integrations: column l of X1 -> M[r][l]
+  if (e == cudaSuccess)
+    e = launch_cfft<false, false>(pad_delay, V, nchan, (int64_t)nchan, (int64_t)1, X1, (int64_t)pad_delay, (int64_t)1, nsub,
+                                  lease.dev, st);
+  if (e == cudaSuccess)
+    e = launch_cfft<true, true>(pad_rate, (const float2*)X1, nsub, (int64_t)1, (int64_t)pad_delay, M, (int64_t)1,
+                                (int64_t)pad_delay, pad_delay, lease.dev, st);
+  PeakSlot peak = {};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&peak, lease.dev, sizeof(peak), cudaMemcpyDeviceToHost, st);
+  // on an error too: the slot is given back only when nothing in flight writes it
+  const cudaError_t waited = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = waited;
+  if (buf) cudaFreeAsync(buf, st);
+  const int64_t idx = (int64_t)(0xFFFFFFFFu - (uint32_t)(peak.best & 0xFFFFFFFFull));
   if (e == cudaSuccess && (idx < 0 || idx >= count)) e = cudaErrorUnknown;
-  if (e == cudaSuccess) e = cudaMemcpy(&pv, M + idx, sizeof(float2), cudaMemcpyDeviceToHost);
-  cudaFreeAsync(buf, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return CORR_ECUDA;
@@ -165,12 +312,12 @@ extern "C" int corr_fringe_search(const float* dev_vis, int nsub, int nchan, int
   if (peak_rate) *peak_rate = (int)(idx / pad_delay);
   if (peak_lag) *peak_lag = (int)(idx % pad_delay);
   if (peak_amp) {
-    const uint32_t bits = (uint32_t)(key >> 32);
+    const uint32_t bits = (uint32_t)(peak.best >> 32);
     memcpy(peak_amp, &bits, sizeof(float));
   }
   if (peak_value) {
-    peak_value[0] = pv.x;
-    peak_value[1] = pv.y;
+    peak_value[0] = peak.value.x;
+    peak_value[1] = peak.value.y;
   }
   return CORR_OK;
 }

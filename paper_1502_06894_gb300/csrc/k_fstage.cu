@@ -73,6 +73,7 @@ cudaError_t fstage_ensure_constants() {
   if (g_const_ctx[dev] != 0 && (id == 0 || g_const_ctx[dev] == id)) return cudaSuccess;
   if ((e = init_w32()) != cudaSuccess) return e;
   if ((e = fstage_pre_init_constants()) != cudaSuccess) return e;
+  if ((e = fringe_init_constants()) != cudaSuccess) return e;
   g_const_ctx[dev] = id ? id : ~0ull;
   return cudaSuccess;
 }
