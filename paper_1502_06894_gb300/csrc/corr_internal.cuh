@@ -145,7 +145,16 @@ cudaError_t launch_fstage(const FParams& p, cudaStream_t s);
 // the pre-F variant (p.pre != 0), nchan <= 4096; launch_fstage dispatches to it
 bool fstage_pre_supported(int nchan);
 cudaError_t launch_fstage_pre(const FParams& p, cudaStream_t s);
+// the F kernels' translation units: launchers by size, and each unit's own constant tables
+cudaError_t launch_fstage_small(const FParams& p, cudaStream_t s);
+cudaError_t launch_fstage_1024(const FParams& p, cudaStream_t s);
+cudaError_t launch_fstage_large(const FParams& p, cudaStream_t s);
+cudaError_t launch_fstage_pre_large(const FParams& p, cudaStream_t s);
+cudaError_t fstage_small_init_constants();
+cudaError_t fstage_1024_init_constants();
+cudaError_t fstage_large_init_constants();
 cudaError_t fstage_pre_init_constants();
+cudaError_t fstage_pre_large_init_constants();
 cudaError_t fringe_init_constants();
 int xstage_kz(int CB, int S, int G, int nchan);
 cudaError_t launch_xstage(const XParams& p, cudaStream_t s);

@@ -72,7 +72,9 @@ cudaError_t fstage_ensure_constants() {
   // id 0 (no context id available): load once per device
   if (g_const_ctx[dev] != 0 && (id == 0 || g_const_ctx[dev] == id)) return cudaSuccess;
   if ((e = init_w32()) != cudaSuccess) return e;
-  if ((e = fstage_pre_init_constants()) != cudaSuccess) return e;
+  for (auto init : {fstage_small_init_constants, fstage_1024_init_constants, fstage_large_init_constants,
+                    fstage_pre_init_constants, fstage_pre_large_init_constants})
+    if ((e = init()) != cudaSuccess) return e;
   if ((e = fringe_init_constants()) != cudaSuccess) return e;
   g_const_ctx[dev] = id ? id : ~0ull;
   return cudaSuccess;
@@ -374,15 +376,6 @@ cudaError_t launch_fstage_tc(const FParams& p, const TcTiles& o, cudaStream_t s)
   }
 }
 
-template <int L>
-static cudaError_t launch_L(const FParams& p, cudaStream_t st) {
-  if constexpr (L >= 256) {
-    if (p.G == 16) return launch_LG<L, 16, false>(p, st);
-    if (p.G == 32) return launch_LG<L, 32, false>(p, st);
-  }
-  return launch_LG<L, 0, false>(p, st);
-}
-
 bool fstage_supported(int nchan) {
   switch (nchan) {
     case 4: case 8: case 16: case 32: case 64: case 128: case 256: case 512:
@@ -396,21 +389,9 @@ bool fstage_supported(int nchan) {
 cudaError_t launch_fstage(const FParams& p, cudaStream_t s) {
   if (p.CB <= 0) return cudaSuccess;
   if (p.pre) return launch_fstage_pre(p, s);
-  switch (p.nchan) {
-    case 4: return launch_L<4>(p, s);
-    case 8: return launch_L<8>(p, s);
-    case 16: return launch_L<16>(p, s);
-    case 32: return launch_L<32>(p, s);
-    case 64: return launch_L<64>(p, s);
-    case 128: return launch_L<128>(p, s);
-    case 256: return launch_L<256>(p, s);
-    case 512: return launch_L<512>(p, s);
-    case 1024: return launch_L<1024>(p, s);
-    case 2048: return launch_L<2048>(p, s);
-    case 4096: return launch_L<4096>(p, s);
-    case 8192: return launch_L<8192>(p, s);
-    default: return cudaErrorInvalidValue;
-  }
+  // the instantiations are split over translation units, which compile side by side
+  if (p.nchan <= 512) return launch_fstage_small(p, s);
+  return p.nchan == 1024 ? launch_fstage_1024(p, s) : launch_fstage_large(p, s);
 }
 
 }  // namespace corr

@@ -8,6 +8,7 @@
 #include <cuda_fp8.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <math.h>
 
 namespace corr {
@@ -69,8 +70,12 @@ template <int P>
 __device__ __forceinline__ int padp(int i) { return i + (i >> ilog2c(P)); }
 
 // In-register DFT of R points (R <= 32): radix-2 decimation in frequency,
-// natural-order input, output permuted back to natural order.  Butterflies
-// with the twiddle -i rotate the difference by a swap and a sign pair.
+// natural-order input, output permuted back to natural order.  A difference
+// whose twiddle is -i stays unrotated: the next stage adds it through the
+// multiply-add that its butterfly needs anyway (the product by +-1 is exact, so
+// the rounding is that of the rotation and the addition), which takes 228
+// packed instructions for 32 points instead of 243, the bound of this routine
+// (two cycles each: 491 -> 460 cycles).
 template <int R>
 __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
   constexpr int LOG = ilog2c(R);
@@ -82,15 +87,13 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
 #pragma unroll
       for (int k = 0; k < half; ++k) {
         const float2 a = v[i + k], b = v[i + k + half];
-        v[i + k] = f2add(a, b);
-        const float2 d = f2sub(a, b);
+        // the first element of a group of differences: b stands for -i b
+        const bool turned = st > 0 && k == 0 && ((i / (2 * half)) & 1);
+        const float2 pm = make_float2(1.f, -1.f), mp = make_float2(-1.f, 1.f);
+        v[i + k] = turned ? f2fma(swp(b), pm, a) : f2add(a, b);
+        const float2 d = turned ? f2fma(swp(b), mp, a) : f2sub(a, b);
         const int m = k * (32 / (2 * half));  // W_{2 half}^k = W_32^m
-        if (m == 0)
-          v[i + k + half] = d;
-        else if (m == 8)
-          v[i + k + half] = f2mul(swp(d), make_float2(1.f, -1.f));  // -i d
-        else
-          v[i + k + half] = cmul_w32(d, m);
+        v[i + k + half] = (m == 0 || m == 8) ? d : cmul_w32(d, m);
       }
     }
   }
@@ -174,11 +177,13 @@ __device__ __forceinline__ void twiddle_products(float2 (&v)[R], const float2 (&
 // reads its points and waits at the barrier.  With s_twp (transforms of
 // 2048+ points) the powers come from a shared table [i][k] of the pass
 // instead: consecutive k in consecutive words, read after the barrier.
-template <int L, int R, int NS, int T, int P, int TWS = 2>
-__device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, int grp,
-                                              const float2* __restrict__ twN,
-                                              const float2* __restrict__ s_twl = nullptr,
-                                              const float2* __restrict__ s_twp = nullptr) {
+//
+// stockham_values leaves the results of butterfly group j = t + uT, point
+// (j / NS) NS R + (j mod NS) + r NS, in v[u][r].
+template <int L, int R, int NS, int T, int P, int TWS>
+__device__ __forceinline__ void stockham_values(const float2* __restrict__ buf, int t, int grp,
+                                                const float2* __restrict__ twN, const float2* __restrict__ s_twl,
+                                                const float2* __restrict__ s_twp, float2 (&v)[L / R / T][R]) {
   constexpr int GROUPS = L / R;
   constexpr int PER = GROUPS / T;
   constexpr int LOGR = ilog2c(R);
@@ -194,7 +199,6 @@ __device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, i
       for (int i = 0; i < LOGR; ++i) wp[u][i] = __ldg(&twN[TWS * k * (1 << i) * (L / (NS * R))]);
     }
   }
-  float2 v[PER][R];
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int j = t + u * T;
@@ -204,8 +208,7 @@ __device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, i
   gsync<T>(grp);
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
-    const int j = t + u * T;
-    const int k = j & (NS - 1);
+    const int k = (t + u * T) & (NS - 1);
     if (tab) {
 #pragma unroll
       for (int r = 1; r < R; ++r) v[u][r] = cmul(v[u][r], s_twl[r * NS + k]);
@@ -217,7 +220,21 @@ __device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, i
       twiddle_products<R, LOGR>(v[u], wp[u]);
     }
     dft_reg<R>(v[u]);
-    const int idxD = (j / NS) * NS * R + k;
+  }
+}
+
+template <int L, int R, int NS, int T, int P, int TWS = 2>
+__device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, int grp,
+                                              const float2* __restrict__ twN,
+                                              const float2* __restrict__ s_twl = nullptr,
+                                              const float2* __restrict__ s_twp = nullptr) {
+  constexpr int PER = L / R / T;
+  float2 v[PER][R];
+  stockham_values<L, R, NS, T, P, TWS>(buf, t, grp, twN, s_twl, s_twp, v);
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int j = t + u * T;
+    const int idxD = (j / NS) * NS * R + (j & (NS - 1));
 #pragma unroll
     for (int r = 0; r < R; ++r) buf[padp<P>(idxD + r * NS)] = v[u][r];
   }
@@ -321,11 +338,7 @@ template <int L> struct LastRadix {
 // transform:  X[k] = E + W O,  X[L-k] = conj(E - W O),  W = W_N^k.  Z is the
 // transform of the halved samples, so E = Z[k] + conj Z[L-k] and
 // O = -i (Z[k] - conj Z[L-k]) carry the split's factor 1/2.
-template <int L, int R0>
-__device__ __forceinline__ void split_pair(const float2* __restrict__ fbuf, float2 w, int k, int km, float2& Xa,
-                                           float2& Xb) {
-  const float2 Zk = fbuf[padp<R0>(k)];
-  const float2 Zm = fbuf[padp<R0>(km)];
+__device__ __forceinline__ void split_values(float2 Zk, float2 Zm, float2 w, float2& Xa, float2& Xb) {
   const float2 pm = make_float2(1.f, -1.f), mp = make_float2(-1.f, 1.f);
   const float2 E = f2fma(Zm, pm, Zk);             // (Zk.x + Zm.x, Zk.y - Zm.y)
   const float2 Ec = f2fma(Zk, pm, Zm);            // conj E
@@ -333,6 +346,12 @@ __device__ __forceinline__ void split_pair(const float2* __restrict__ fbuf, floa
   const float2 WO = cmul(O, w);
   Xa = f2add(E, WO);
   Xb = f2fma(WO, mp, Ec);                         // (E.x - WO.x, WO.y - E.y)
+}
+
+template <int L, int R0>
+__device__ __forceinline__ void split_pair(const float2* __restrict__ fbuf, float2 w, int k, int km, float2& Xa,
+                                           float2& Xb) {
+  split_values(fbuf[padp<R0>(k)], fbuf[padp<R0>(km)], w, Xa, Xb);
 }
 
 // The split's twiddles W_N^k along a thread's channels k = t + qT: from the
@@ -441,6 +460,42 @@ __device__ __forceinline__ void split_rotate_store(const float2* __restrict__ fb
   }
 }
 
+// Split, rotate and store from the registers of one warp's transform.  Z[L - k]
+// of k = t + qT is element Q - 1 - q of thread T - t (element Q - q of thread 0
+// itself), so half the values cross lanes by shuffles, where the shared-memory
+// form writes and reads all of them: 32 shared-memory cycles a 1024-point
+// transform instead of 128.
+template <int L, int T, int OUT, int PER, int R>
+__device__ __forceinline__ void split_rotate_shuffle(const float2 (&z_)[PER][R], const float2* __restrict__ s_tw, int t,
+                                                     float phi, float delta, void* out, size_t obase, float scale) {
+  constexpr int Q = L / T;
+  static_assert(PER * R == Q, "last pass");
+  auto v = [&](int q) { return z_[q % PER][q / PER]; };  // Z[t + q T]
+  const unsigned mask = T == 32 ? 0xffffffffu : ((1u << T) - 1u) << (threadIdx.x & 31u & ~(unsigned)(T - 1));
+  const int partner = (T - t) & (T - 1);
+  float2 z = cis_turns(fmaf((float)t, delta, phi));
+  float2 y = cis_turns(fmaf((float)(L - t), delta, phi));
+  float cm1, sn;
+  walk_step((float)T * delta, cm1, sn);
+#pragma unroll
+  for (int q = 0; q < Q / 2; ++q) {
+    const int k = t + q * T;
+    const float2 give = t == 0 ? v((Q - q) % Q) : v(Q - 1 - q);
+    const float2 Zm = make_float2(__shfl_sync(mask, give.x, partner, T), __shfl_sync(mask, give.y, partner, T));
+    float2 Xa, Xb;
+    split_values(v(q), Zm, s_tw[L + k], Xa, Xb);
+    store_spec<OUT>(out, obase + k, cmul(Xa, z), scale);
+    if (q > 0 || t != 0) store_spec<OUT>(out, obase + (L - k), cmul(Xb, y), scale);
+    z = walk(z, cm1, sn);
+    y = walk(y, cm1, -sn);
+  }
+  if (t == 0) {  // k = L/2: X = E + W_N^{N/4} O; z has walked to it
+    float2 Xa, Xb;
+    split_values(v(Q / 2), v(Q / 2), make_float2(0.f, -1.f), Xa, Xb);
+    store_spec<OUT>(out, obase + L / 2, cmul(Xa, z), scale);
+  }
+}
+
 // Byte offset of the packed-word staging area after the NGRP FFT buffers,
 // rounded up to 16 bytes for the 16-byte shared-memory stores.
 template <int L>
@@ -475,9 +530,9 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 // Stage the packed windows of `nslots` blocks (chunk blocks bb0...) into
-// wbuf (slot stride wslot words) with asynchronous copies from device memory
-// (plain loads from pinned host memory): 16-byte copies where the words lie
-// inside the station's data, single words at its end.
+// wbuf (slot stride wslot words) with asynchronous copies (plain loads from
+// pinned host memory unless ASYNC): 16-byte copies where the words lie inside
+// the station's data, single words at its end.
 // The copy of slot sl starts at the 16-byte aligned word a0 = w0 & ~3; with
 // GC = 16 (one word per sample time) word w0 goes to an even index so that
 // every sample pair is one aligned 64-bit load (odd leads are copied word by
@@ -486,11 +541,15 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // pair is one aligned 16-byte load (a lead of 2 is copied in 8-byte pieces,
 // two words further on).  s_ok / s_boff receive each slot's validity and the
 // bit offset of its window from the slot's first word.
-template <int N, int GC>
+template <int N, int GC, bool ASYNC>
 __device__ __forceinline__ void stage_windows(const FParams& p, const StationView& sv, int s, int G, int bb0,
                                               int nslots, uint32_t* wbuf, int wslot, int* s_ok, int* s_boff) {
-  const int tid = threadIdx.x;
-  for (int sl = 0; sl < nslots; ++sl) {
+  // several windows: a share of the warps each, so that their descriptor
+  // loads (and the copies behind them) run side by side, not one after another
+  const int ways = min(nslots, (int)(blockDim.x >> 5));
+  const int nt = (int)(blockDim.x / ways) & ~31;  // threads per window
+  const int tid = threadIdx.x % nt, way = threadIdx.x / nt;
+  for (int sl = way < ways ? way : nslots; sl < nslots; sl += ways) {
     const int d = p.blk0 + bb0 + sl;
     const bool ok = p.valid[(size_t)s * p.ld + d] != 0;
     int64_t w0 = 0;
@@ -511,11 +570,13 @@ __device__ __forceinline__ void stage_windows(const FParams& p, const StationVie
     const int64_t a0 = w0 - lead;
     const int ntot = nw + lead;
     const int nvec = ntot >> 2;
-    if (sv.host) {
-      // pinned host memory over the host link: plain 16-byte loads (they
-      // keep more of the link's requests in flight than the async copies)
+    if (!ASYNC && sv.host) {
+      // pinned host memory over the host link: plain 16-byte loads keep more
+      // of the link's requests in flight than the async copies, which matters
+      // while the CTA waits for its windows (with ASYNC they pass behind a
+      // whole step of transforms)
       const uint4* src4 = reinterpret_cast<const uint4*>(sv.words + a0);
-      for (int q = tid; q < nvec; q += blockDim.x) {
+      for (int q = tid; q < nvec; q += nt) {
         if (a0 + 4 * q + 4 <= sv.nwords) {
           const uint4 x = __ldg(src4 + q);
           if (shift) {
@@ -531,10 +592,10 @@ __device__ __forceinline__ void stage_windows(const FParams& p, const StationVie
             if (a0 + 4 * q + u < sv.nwords) dst[4 * q + u] = __ldg(&sv.words[a0 + 4 * q + u]);
         }
       }
-      for (int q = 4 * nvec + tid; q < ntot; q += blockDim.x)
+      for (int q = 4 * nvec + tid; q < ntot; q += nt)
         if (a0 + q < sv.nwords) dst[q] = __ldg(&sv.words[a0 + q]);
     } else {
-      for (int q = tid; q < nvec; q += blockDim.x) {
+      for (int q = tid; q < nvec; q += nt) {
         if (a0 + 4 * q + 4 <= sv.nwords) {
           if (shift == 2) {
             cp_async8(dst + 4 * q, sv.words + a0 + 4 * q);
@@ -550,7 +611,7 @@ __device__ __forceinline__ void stage_windows(const FParams& p, const StationVie
             if (a0 + 4 * q + u < sv.nwords) cp_async4(dst + 4 * q + u, sv.words + a0 + 4 * q + u);
         }
       }
-      for (int q = 4 * nvec + tid; q < ntot; q += blockDim.x)
+      for (int q = 4 * nvec + tid; q < ntot; q += nt)
         if (a0 + q < sv.nwords) cp_async4(dst + q, sv.words + a0 + q);
     }
     if (tid == 0) {
@@ -587,13 +648,160 @@ __device__ __forceinline__ void load_pair(const uint32_t* __restrict__ wsl, int 
   }
 }
 
+// Transpose a 16 x 16 matrix of 2-bit fields: field i of word j becomes field
+// j of word i.
+__device__ __forceinline__ void transpose_fields(uint32_t (&a)[16]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const uint32_t x = a[i], y = a[i + 8];
+    a[i] = __byte_perm(x, y, 0x5410);
+    a[i + 8] = __byte_perm(x, y, 0x7632);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = (q & 3) + 2 * (q & 4);
+    const uint32_t x = a[i], y = a[i + 4];
+    a[i] = __byte_perm(x, y, 0x6240);
+    a[i + 4] = __byte_perm(x, y, 0x7351);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = (q & 1) + 2 * (q & 6);
+    const uint32_t x = a[i], y = a[i + 2], m = 0x0F0F0F0Fu;
+    a[i] = (x & m) | ((y << 4) & ~m);
+    a[i + 2] = ((x >> 4) & m) | (y & ~m);
+  }
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int i = 2 * q;
+    const uint32_t x = a[i], y = a[i + 1], m = 0x33333333u;
+    a[i] = (x & m) | ((y << 2) & ~m);
+    a[i + 1] = ((x >> 2) & m) | (y & ~m);
+  }
+}
+
+// The first pass's codes, stream by stream.  The staged window interleaves the
+// streams, so that each transform had to read all of it: 32 64-bit loads and
+// as many shifts and masks a thread for a 1024-point transform, an eighth of
+// the kernel's shared-memory traffic.  Here the CTA turns the window once for
+// all streams: thread t of a transform takes points t + r T, r < R0, whose
+// codes (two samples a point; one in the pre-F form) become the 2-bit fields
+// of W words, [slot][stream][word][thread], read as W consecutive loads.
+template <int L, bool PRE> struct Codes {
+  static constexpr int T = Plan<L>::T, R0 = Plan<L>::R0;
+  static constexpr int F = R0 * (PRE ? 1 : 2);   // fields per thread
+  static constexpr int W = (F + 15) / 16;
+  static constexpr bool on = L >= 64 && L <= 4096 && L / R0 == T;  // one point group a thread
+};
+
+// One stream (post-F form): the window is a row of 4-bit point codes, and the
+// words of eight threads come from an 8 x 8 transpose of them.
+template <int L>
+__device__ __forceinline__ void turn_codes_one(const uint32_t* __restrict__ wbuf, int wslot, const int* s_ok,
+                                               const int* s_boff, int nslots, uint32_t* codes) {
+  using C = Codes<L, false>;
+  constexpr int T = C::T, W = C::W;
+  for (int e = threadIdx.x; e < nslots * W * (T / 8); e += blockDim.x) {
+    const int t8 = e % (T / 8);
+    const int w = e / (T / 8) % W;
+    const int sl = e / (T / 8) / W;
+    if (!s_ok[sl]) continue;
+    const int boff = s_boff[sl];
+    const uint32_t* wsl = wbuf + sl * wslot;
+    uint32_t a[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {  // points 8 t8 .. 8 t8 + 7 of row r = 8 w + i
+      const int bit = boff + 4 * (8 * t8 + (8 * w + i) * T);
+      a[i] = __funnelshift_r(wsl[bit >> 5], wsl[(bit >> 5) + 1], bit & 31);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t x = a[i], y = a[i + 4];
+      a[i] = __byte_perm(x, y, 0x5410);
+      a[i + 4] = __byte_perm(x, y, 0x7632);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = (q & 1) + 2 * (q & 2);
+      const uint32_t x = a[i], y = a[i + 2];
+      a[i] = __byte_perm(x, y, 0x6240);
+      a[i + 2] = __byte_perm(x, y, 0x7351);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = 2 * q;
+      const uint32_t x = a[i], y = a[i + 1], m = 0x0F0F0F0Fu;
+      a[i] = (x & m) | ((y << 4) & ~m);
+      a[i + 1] = ((x >> 4) & m) | (y & ~m);
+    }
+    uint4* dst = reinterpret_cast<uint4*>(codes + (sl * W + w) * T + 8 * t8);
+    dst[0] = make_uint4(a[0], a[1], a[2], a[3]);
+    dst[1] = make_uint4(a[4], a[5], a[6], a[7]);
+  }
+}
+
+// Streams [j0, j0 + jb) of `nslots` staged windows into `codes`.
+template <int L, int GC, bool PRE>
+__device__ __forceinline__ void turn_codes(const uint32_t* __restrict__ wbuf, int wslot, const int* s_ok,
+                                           const int* s_boff, int nslots, int G, int j0, int jb, uint32_t* codes) {
+  using C = Codes<L, PRE>;
+  constexpr int T = C::T, W = C::W, F = C::F;
+  if constexpr (GC == 0 && !PRE && T >= 8) {
+    if (G == 1) return turn_codes_one<L>(wbuf, wslot, s_ok, s_boff, nslots, codes);
+  }
+  const int halves = (jb + 15) >> 4;  // 16 streams at a time
+  for (int e = threadIdx.x; e < nslots * halves * W * T; e += blockDim.x) {
+    const int t = e % T;
+    int q = e / T;
+    const int w = q % W;
+    q /= W;
+    const int sl = q / halves, h = q - sl * halves;
+    if (!s_ok[sl]) continue;
+    const int boff = s_boff[sl];
+    const uint32_t* wsl = wbuf + sl * wslot + (GC ? (boff >> 5) : 0);
+    uint32_t a[16];
+#pragma unroll
+    for (int f = 0; f < 16; f += PRE ? 1 : 2) {
+      const int fi = 16 * w + f;
+      const int m = t + (PRE ? fi : fi >> 1) * T;  // point
+      if (F < 16 && f >= F) {
+        a[f] = 0u;
+        if (!PRE) a[f + 1] = 0u;
+      } else if constexpr (GC == 16 && PRE) {
+        a[f] = wsl[m];
+      } else if constexpr (GC == 16) {  // the staging put the window's first word at an even index
+        const uint2 x = *reinterpret_cast<const uint2*>(wsl + 2 * m);
+        a[f] = x.x;
+        a[f + 1] = x.y;
+      } else if constexpr (GC == 32 && PRE) {
+        a[f] = wsl[2 * m + (j0 >> 4) + h];
+      } else if constexpr (GC == 32) {
+        a[f] = wsl[4 * m + (j0 >> 4) + h];
+        a[f + 1] = wsl[4 * m + 2 + (j0 >> 4) + h];
+      } else {
+        const int bit = boff + 2 * ((PRE ? m : 2 * m) * G + j0 + 16 * h);
+        a[f] = __funnelshift_r(wsl[bit >> 5], wsl[(bit >> 5) + 1], bit & 31);
+        if constexpr (!PRE) {
+          const int bit1 = bit + 2 * G;
+          a[f + 1] = G <= 8 ? a[f] >> (2 * G) : __funnelshift_r(wsl[bit1 >> 5], wsl[(bit1 >> 5) + 1], bit1 & 31);
+        }
+      }
+    }
+    transpose_fields(a);
+    uint32_t* dst = codes + ((size_t)(sl * jb + 16 * h) * W + w) * T + t;
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+      if (16 * h + j < jb) dst[j * W * T] = a[j];
+  }
+}
+
 // CTAs per SM the register allocation must allow: larger FFTs run one group
 // of 128-256 threads per FFT, so without a bound the compiler takes up to
 // 255 registers and a single CTA fills the SM's register file.  (4096- and
 // 8192-point transforms keep one CTA of 512 / 256 threads per SM: their
 // buffers and staged windows fill shared memory anyway.)
 template <int L> struct MinBlocks {
-  static constexpr int v = (L >= 512 && L <= 1024) ? 2 : (L == 2048 ? 3 : 1);
+  static constexpr int v = (L >= 64 && L <= 1024) ? 2 : (L == 2048 ? 3 : 1);
 };
 // the tensor-core F step keeps its 8 groups' spectra in shared memory
 template <int L> struct MinBlocksTC {
@@ -641,24 +849,24 @@ __device__ __forceinline__ float2 prerot(int m, float phi0, float dhi, float dlo
 // Store of the pre-F path: channels k = 0..L/2-1 of the complex L-point
 // transform, times the fractional-delay slope exp(+2 pi i k delta) (the
 // fringe phase was applied before the transform), by the same walk as the
-// post-F store.
-template <int L, int T, int R0, int OUT>
-__device__ __forceinline__ void rotate_store_pre(const float2* __restrict__ fbuf, int t, bool ok, float delta,
-                                                 void* out, size_t obase, float scale) {
+// post-F store.  v(q) is Z[t + qT]: the thread's own results of the last pass,
+// which need not pass through shared memory.
+template <int L, int T, int OUT>
+__device__ __forceinline__ void store_zeros_pre(int t, void* out, size_t obase) {
+#pragma unroll 4
+  for (int q = 0; q < L / 2 / T; ++q) store_spec<OUT>(out, obase + t + q * T, make_float2(0.f, 0.f), 1.f);
+}
+
+template <int L, int T, int OUT, typename V>
+__device__ __forceinline__ void rotate_store_pre(V v, int t, float delta, void* out, size_t obase, float scale) {
   constexpr int Q = (L / 2) / T;
   static_assert(Q >= 1 && (L / 2) % T == 0, "plan");
-  if (!ok) {
-#pragma unroll 4
-    for (int q = 0; q < Q; ++q) store_spec<OUT>(out, obase + t + q * T, make_float2(0.f, 0.f), scale);
-    return;
-  }
   float2 z = cis_turns((float)t * delta);
   float cm1, sn;
   walk_step((float)T * delta, cm1, sn);
-#pragma unroll 4
+#pragma unroll
   for (int q = 0; q < Q; ++q) {
-    const int k = t + q * T;
-    store_spec<OUT>(out, obase + k, cmul(fbuf[padp<R0>(k)], z), scale);
+    store_spec<OUT>(out, obase + t + q * T, cmul(v(q), z), scale);
     z = walk(z, cm1, sn);
   }
 }
@@ -667,10 +875,18 @@ __device__ __forceinline__ void rotate_store_pre(const float2* __restrict__ fbuf
 // L-point complex transform (even/odd samples packed), real split, post-F
 // rotation.  PRE = true: the N = L real samples rotated one by one by the
 // fringe phase into an L-point complex transform, then the fractional-delay
-// slope.
-template <int L, int GC, bool PRE>
+// slope.  TURN: the codes come stream by stream from turn_codes, jb streams at
+// a time; else each transform decodes the staged window itself.
+//
+// Bound by the mix of the FMA pipe (48%), the shared-memory pipe (54%) and
+// instruction issue (52%) at the 16 warps that 32 points a thread leave an SM:
+// no one of its parts, taken out, gives more than 9%.  Ten stations x 16
+// streams x 1024 channels, 819 blocks (2.7e8 samples): 328 us; 376 us when each
+// transform decoded the interleaved window (shared-memory pipe 71%) and passed
+// its last pass through shared memory again.
+template <int L, int GC, bool PRE, bool TURN>
 __global__ void __launch_bounds__(Groups<L>::T * Groups<L>::NGRP, MinBlocks<L>::v)
-k_fstage(FParams p, int slots, int wslot, int nseq) {
+k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
   using P = Plan<L>;
   constexpr int T = P::T;
   constexpr int NGRP = Groups<L>::NGRP;
@@ -679,12 +895,16 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
   constexpr int BUF = kBufPad<L>();
   constexpr int R0 = P::R0;
   constexpr int PER0 = L / R0 / T;
+  // the last pass's results stay in registers: the pre-F form's store needs only a thread's own,
+  // the real split those of another thread, which a shuffle reaches within a warp
+  constexpr bool REGS = PRE || (T <= 32 && Tw<L>::on && P::R1 > 1 && P::R2 == 1);
   static_assert(PER0 >= 1, "plan");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* fbuf_all = reinterpret_cast<float2*>(smem_raw);
   static_assert(kWordsOffset<L>(NGRP) % 16 == 0, "staging area must be 16-byte aligned");
   uint32_t* wbuf = reinterpret_cast<uint32_t*>(smem_raw + kWordsOffset<L>(NGRP));
+  uint32_t* codes = wbuf + slots * wslot;  // TURN
 
   const int tid = threadIdx.x;
   const int grp = tid / T;
@@ -695,8 +915,9 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
   const StationView sv = p.st[s];
 
   // this CTA: nseq steps of `slots` blocks each, from chunk block `first`;
-  // with nseq > 1 the windows of step it+1 are copied (asynchronously, into
-  // the other half of a double buffer) while step it is transformed
+  // the windows of step it+1 are copied asynchronously while step it is
+  // transformed: into the staging area itself once its codes are turned, else
+  // into the other half of a double buffer
   const int first = blockIdx.x * nseq * slots;
   if (first >= p.CB) return;
 
@@ -708,27 +929,44 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
   fill_tables<L, LastRadix<L>::v, TWS>(s_lut16, s_tw, p);
   fill_pass_tables<L, TWS>(s_twp, p.twN);
 
-  stage_windows<N, GC>(p, sv, s, G, first, min(slots, p.CB - first), wbuf, wslot, s_ok[0], s_boff[0]);
+  stage_windows<N, GC, false>(p, sv, s, G, first, min(slots, p.CB - first), wbuf, wslot, s_ok[0], s_boff[0]);
   cp_async_commit();
   for (int it = 0; it < nseq; ++it) {
     const int bb0 = first + it * slots;
     if (bb0 >= p.CB) break;  // uniform over the CTA
     const int nslots = min(slots, p.CB - bb0);
     const int nb = it & 1;
-    if (it + 1 < nseq && bb0 + slots < p.CB)
-      stage_windows<N, GC>(p, sv, s, G, bb0 + slots, min(slots, p.CB - bb0 - slots), wbuf + (nb ^ 1) * slots * wslot,
-                           wslot, s_ok[nb ^ 1], s_boff[nb ^ 1]);
-    cp_async_commit();
-    cp_async_wait<1>();  // this step's windows have landed (the next step's may still fly)
+    const bool more = it + 1 < nseq && bb0 + slots < p.CB;
+    uint32_t* wcur = wbuf;
+    if constexpr (TURN) {
+      cp_async_wait<0>();
+    } else {
+      wcur = wbuf + nb * slots * wslot;
+      if (more)
+        stage_windows<N, GC, TURN>(p, sv, s, G, bb0 + slots, min(slots, p.CB - bb0 - slots), wbuf + (nb ^ 1) * slots * wslot,
+                             wslot, s_ok[nb ^ 1], s_boff[nb ^ 1]);
+      cp_async_commit();
+      cp_async_wait<1>();  // this step's windows have landed (the next step's may still fly)
+    }
     __syncthreads();
-    uint32_t* wcur = wbuf + nb * slots * wslot;
 
-    const int ntasks = nslots * G;
+    for (int j0 = 0; j0 < G; j0 += jb) {
+    const int nj = min(jb, G - j0);
+    if constexpr (TURN) {
+      turn_codes<L, GC, PRE>(wcur, wslot, s_ok[nb], s_boff[nb], nslots, G, j0, nj, codes);
+      __syncthreads();
+      if (more && j0 + jb >= G) {  // the window has been read
+        stage_windows<N, GC, TURN>(p, sv, s, G, bb0 + slots, min(slots, p.CB - bb0 - slots), wbuf, wslot, s_ok[nb ^ 1],
+                             s_boff[nb ^ 1]);
+        cp_async_commit();
+      }
+    }
+    const int ntasks = nslots * nj;
     for (int base = 0; base < ntasks; base += NGRP) {
       const int task = base + grp;
       const bool active = task < ntasks;
-      const int sl = active ? task / G : 0;
-      const int j = active ? task - sl * G : 0;
+      const int sl = active ? task / nj : 0;
+      const int j = active ? j0 + task - sl * nj : 0;
       const bool ok = active && s_ok[nb][sl];
       const int boff = s_boff[nb][sl];
       // for GC = 16 / 32 the window starts on a word boundary: skip the lead
@@ -739,10 +977,17 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
       // during the transform
       const float delta = ok ? p.delta[(size_t)s * p.ld + d] : 0.f;
       const float phi = (ok && !PRE) ? p.phi[((size_t)s * p.nsub + j / p.npol) * p.ld + d] : 0.f;
+      constexpr int NCH = PRE ? L / 2 : L;
+      const size_t obase = spec_row(p, j, bb0 + sl, s) * (size_t)NCH;
 
       // ---- pass 0: unpack straight into registers (NS = 1, no twiddles);
       //      the transform of a block that is not valid is skipped ----
       if (ok) {
+        uint32_t cw[Codes<L, PRE>::W];
+        if constexpr (TURN) {
+#pragma unroll
+          for (int w = 0; w < Codes<L, PRE>::W; ++w) cw[w] = codes[(task * Codes<L, PRE>::W + w) * T + t];
+        }
         float2 v[PER0][R0];
         if constexpr (PRE) {
           const size_t ps = ((size_t)s * p.nsub + j / p.npol) * p.ld + d;
@@ -754,8 +999,9 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
 #pragma unroll
             for (int r = 0; r < R0; ++r) {
               const int m = jj + r * (L / R0);
+              const uint32_t c = TURN ? (cw[r >> 4] >> (2 * (r & 15))) & 3u : load_one<GC>(wsl, boff, G, m, j);
               // s_lut16[c] = (l[c] / 2, l[0] / 2): twice its real part is level c
-              const float lev = 2.0f * s_lut16[load_one<GC>(wsl, boff, G, m, j)].x;
+              const float lev = 2.0f * s_lut16[c].x;
               const float2 z = prerot(m, phi0, dph.x, dph.y);
               v[u][r] = f2mul(z, bc(lev));
             }
@@ -766,10 +1012,13 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
             const int jj = t + u * T;
 #pragma unroll
             for (int r = 0; r < R0; ++r) {
-              const int m = jj + r * (L / R0);
-              uint32_t c0, c1;
-              load_pair<GC>(wsl, boff, G, m, j, c0, c1);
-              v[u][r] = s_lut16[c0 | (c1 << 2)];
+              if constexpr (TURN) {
+                v[u][r] = s_lut16[(cw[r >> 3] >> (4 * (r & 7))) & 15u];
+              } else {
+                uint32_t c0, c1;
+                load_pair<GC>(wsl, boff, G, jj + r * (L / R0), j, c0, c1);
+                v[u][r] = s_lut16[c0 | (c1 << 2)];
+              }
             }
           }
         }
@@ -777,78 +1026,133 @@ k_fstage(FParams p, int slots, int wslot, int nseq) {
         for (int u = 0; u < PER0; ++u) {
           const int jj = t + u * T;
           dft_reg<R0>(v[u]);
+          if constexpr (P::R1 > 1 || !REGS) {
 #pragma unroll
-          for (int r = 0; r < R0; ++r) fbuf[padp<R0>(jj * R0 + r)] = v[u][r];
+            for (int r = 0; r < R0; ++r) fbuf[padp<R0>(jj * R0 + r)] = v[u][r];
+          }
         }
-        gsync<T>(grp);
-        if constexpr (P::R1 > 1)
-          stockham_pass<L, P::R1, P::R0, T, P::R0, TWS>(fbuf, t, grp, p.twN, Tw<L>::on ? s_tw : nullptr,
-                                                        PassTw<L>::on ? s_twp : nullptr);
-        if constexpr (P::R2 > 1)
-          stockham_pass<L, P::R2, P::R0 * P::R1, T, P::R0, TWS>(fbuf, t, grp, p.twN, nullptr,
-                                                                PassTw<L>::on ? s_twp + PassTw<L>::n1 : nullptr);
+        // the passes after the first; the last one's results stay in registers
+        // where their thread (pre-F) or warp (post-F) can finish them
+        constexpr int RL = LastRadix<L>::v, PERL = L / RL / T;
+        const float2* twl = Tw<L>::on ? s_tw : nullptr;
+        const float2* twp1 = PassTw<L>::on ? s_twp : nullptr;
+        const float2* twp2 = PassTw<L>::on ? s_twp + PassTw<L>::n1 : nullptr;
+        if constexpr (P::R1 > 1) gsync<T>(grp);
+        if constexpr (P::R2 > 1) stockham_pass<L, P::R1, P::R0, T, P::R0, TWS>(fbuf, t, grp, p.twN, nullptr, twp1);
+        if constexpr (REGS) {
+          float2 z[PERL][RL];
+          if constexpr (P::R1 > 1) {
+            stockham_values<L, RL, L / RL, T, P::R0, TWS>(fbuf, t, grp, p.twN, twl, P::R2 > 1 ? twp2 : twp1, z);
+            // Z[t + q T] = z[q % PERL][q / PERL]
+          } else {
+#pragma unroll
+            for (int r = 0; r < RL; ++r) z[0][r] = v[0][r];
+          }
+          auto finish = [&](auto kind) {
+            constexpr int OUT = decltype(kind)::value;
+            if constexpr (PRE)
+              rotate_store_pre<L, T, OUT>([&](int q) { return z[q % PERL][q / PERL]; }, t, delta, p.out, obase, p.scale);
+            else
+              split_rotate_shuffle<L, T, OUT>(z, s_tw, t, phi, delta, p.out, obase, p.scale);
+          };
+          if (p.out_kind == 1) finish(std::integral_constant<int, 1>{});
+          else if (p.out_kind == 2) finish(std::integral_constant<int, 2>{});
+          else finish(std::integral_constant<int, 0>{});
+        } else if constexpr (P::R1 > 1) {
+          stockham_pass<L, RL, L / RL, T, P::R0, TWS>(fbuf, t, grp, p.twN, twl, P::R2 > 1 ? twp2 : twp1);
+        } else {
+          gsync<T>(grp);
+        }
       }
 
-      // ---- store (real split and post-F rotation, or the pre-F path's slope) ----
-      if (active) {
-        const int bb = bb0 + sl;
+      // ---- store (real split and post-F rotation, or the pre-F path's
+      //      slope); a block that is not valid stores zeros ----
+      if (active && !(REGS && ok)) {
         if constexpr (PRE) {
-          constexpr int NCH = L / 2;
-          const size_t obase = spec_row(p, j, bb, s) * (size_t)NCH;
           if (p.out_kind == 1)
-            rotate_store_pre<L, T, R0, 1>(fbuf, t, ok, delta, p.out, obase, p.scale);
+            store_zeros_pre<L, T, 1>(t, p.out, obase);
           else if (p.out_kind == 2)
-            rotate_store_pre<L, T, R0, 2>(fbuf, t, ok, delta, p.out, obase, p.scale);
+            store_zeros_pre<L, T, 2>(t, p.out, obase);
           else
-            rotate_store_pre<L, T, R0, 0>(fbuf, t, ok, delta, p.out, obase, p.scale);
+            store_zeros_pre<L, T, 0>(t, p.out, obase);
         } else {
-          const size_t obase = spec_row(p, j, bb, s) * (size_t)L;
           if (p.out_kind == 1)
-            split_rotate_store<L, T, R0, 1>(fbuf, s_tw, p.twN, t, ok, phi, delta, p.out, obase, p.scale);
+            split_rotate_store<L, T, R0, 1>(fbuf, s_tw, p.twN, t, ok && !REGS, phi, delta, p.out, obase, p.scale);
           else if (p.out_kind == 2)
-            split_rotate_store<L, T, R0, 2>(fbuf, s_tw, p.twN, t, ok, phi, delta, p.out, obase, p.scale);
+            split_rotate_store<L, T, R0, 2>(fbuf, s_tw, p.twN, t, ok && !REGS, phi, delta, p.out, obase, p.scale);
           else
-            split_rotate_store<L, T, R0, 0>(fbuf, s_tw, p.twN, t, ok, phi, delta, p.out, obase, p.scale);
+            split_rotate_store<L, T, R0, 0>(fbuf, s_tw, p.twN, t, ok && !REGS, phi, delta, p.out, obase, p.scale);
         }
       }
       gsync<T>(grp);
     }
-    __syncthreads();  // every read of this step's windows is done before they are overwritten
+    __syncthreads();  // every read of this step's windows and codes is done before they are overwritten
+    }
   }
+}
+
+template <int L, int GC, bool PRE, bool TURN>
+static cudaError_t launch_turn(const FParams& p, int slots, int wslot, int jb, int nseq, size_t smem, cudaStream_t st) {
+  cudaError_t e =
+      cudaFuncSetAttribute(k_fstage<L, GC, PRE, TURN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int per_cta = slots * nseq;
+  dim3 grid((p.CB + per_cta - 1) / per_cta, p.S);
+  k_fstage<L, GC, PRE, TURN><<<grid, Plan<L>::T * Groups<L>::NGRP, smem, st>>>(p, slots, wslot, nseq, jb);
+  return cudaGetLastError();
 }
 
 template <int L, int GC, bool PRE>
 static cudaError_t launch_LG(const FParams& p, cudaStream_t st) {
-  constexpr int T = Plan<L>::T;
   constexpr int NGRP = Groups<L>::NGRP;
   const int N = PRE ? L : 2 * L;
-  int slots = NGRP / p.G;
-  if (slots < 1) slots = 1;
-  if (slots > 64) slots = 64;
   const int wslot = wslot_words(N, p.G);
-  const size_t one = kWordsOffset<L>(NGRP) + (size_t)slots * wslot * sizeof(uint32_t);
-  const size_t two = one + (size_t)slots * wslot * sizeof(uint32_t);
-  // Several steps per CTA (tables filled once, the next windows copied while
-  // the current ones are transformed) when the double buffer still lets the
-  // kernel keep its CTAs per SM and the grid stays at 8+ waves of them.
+  const size_t fixed = sizeof(float2) * (Tw<L>::size + PassTw<L>::size) + 2048;
+  auto resident = [&](size_t smem) { return (int)std::min<size_t>(MinBlocks<L>::v, 227 * 1024 / (smem + fixed)); };
+  auto window = [&](int slots) { return (size_t)slots * wslot * sizeof(uint32_t); };
+  auto turned = [&](int slots, int jb) {
+    return kWordsOffset<L>(NGRP) + window(slots) +
+           sizeof(uint32_t) * (size_t)slots * jb * Codes<L, PRE>::W * Codes<L, PRE>::T;
+  };
   static int sm_count = 0;
   if (!sm_count) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       sm_count = 152;
   }
-  const int64_t steps = (int64_t)((p.CB + slots - 1) / slots) * p.S;
-  int nseq = 1;
-  if ((size_t)MinBlocks<L>::v * (two + sizeof(float2) * (Tw<L>::size + PassTw<L>::size) + 1024) <= 227 * 1024)
-    nseq = (int)std::max<int64_t>(1, std::min<int64_t>(4, steps / ((int64_t)8 * MinBlocks<L>::v * sm_count)));
-  const size_t smem = nseq > 1 ? two : one;
-  if (smem + sizeof(float2) * (Tw<L>::size + PassTw<L>::size) + 1024 > 227 * 1024) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(k_fstage<L, GC, PRE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int per_cta = slots * nseq;
-  dim3 grid((p.CB + per_cta - 1) / per_cta, p.S);
-  k_fstage<L, GC, PRE><<<grid, T * NGRP, smem, st>>>(p, slots, wslot, nseq);
-  return cudaGetLastError();
+  // Steps per CTA.  A start (tables, first windows) costs about a fifth of one
+  // round of transforms, so a CTA whose step is one round takes eight steps
+  // (1024 samples, 8 streams: 412 us against 489 with one step each); from four
+  // rounds a step on, more and shorter CTAs even out the last wave better
+  // (2048 samples, 16 streams: 328 us against 338 with two steps).  At least
+  // four waves stay.
+  auto steps_per_cta = [&](int slots, int ctas) {
+    const int rounds = std::max(1, slots * p.G / NGRP);
+    const int64_t steps = (int64_t)((p.CB + slots - 1) / slots) * p.S;
+    const int64_t most = std::max<int64_t>(1, steps / ((int64_t)4 * ctas * sm_count));
+    return (int)std::min<int64_t>(rounds >= 4 ? 1 : (8 + rounds - 1) / rounds, most);
+  };
+  // blocks a CTA takes at a time: as many as give every group a transform
+  const int base = std::max(1, std::min(64, NGRP / p.G));
+  // Codes turned stream by stream: the turned codes of all streams (of 16 at a
+  // time if more do not fit) beside the windows, as long as they cost no CTA
+  // per SM; two blocks at a time where they fit too (a step ends at a barrier).
+  if constexpr (Codes<L, PRE>::on) {
+    const int most = std::max(1, resident(kWordsOffset<L>(NGRP) + window(base)));
+    if (base == 1 && resident(turned(2, p.G)) >= most && p.CB >= 2)
+      return launch_turn<L, GC, PRE, true>(p, 2, wslot, p.G, steps_per_cta(2, most), turned(2, p.G), st);
+    for (const int jb : {p.G, 16})
+      if (jb <= p.G && resident(turned(base, jb)) >= most)
+        return launch_turn<L, GC, PRE, true>(p, base, wslot, jb, steps_per_cta(base, most), turned(base, jb), st);
+  }
+  if constexpr (!Codes<L, PRE>::on || (L == 2048 && !PRE)) {  // (2048 points, more than 18 streams)
+    const size_t one = kWordsOffset<L>(NGRP) + window(base), two = one + window(base);
+    const int nseq = resident(two) == MinBlocks<L>::v ? steps_per_cta(base, resident(two)) : 1;
+    const size_t smem = nseq > 1 ? two : one;
+    if (resident(smem) < 1) return cudaErrorInvalidConfiguration;
+    return launch_turn<L, GC, PRE, false>(p, base, wslot, p.G, nseq, smem, st);
+  }
+  return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace corr

@@ -18,7 +18,7 @@ cudaError_t fstage_pre_init_constants() { return init_w32(); }
 bool fstage_pre_supported(int nchan) { return nchan >= 4 && nchan <= 4096; }
 
 template <int L>
-static cudaError_t launch_pre_L(const FParams& p, cudaStream_t st) {
+static cudaError_t launch_L(const FParams& p, cudaStream_t st) {
   if constexpr (L >= 256) {
     if (p.G == 16) return launch_LG<L, 16, true>(p, st);
     if (p.G == 32) return launch_LG<L, 32, true>(p, st);
@@ -29,18 +29,14 @@ static cudaError_t launch_pre_L(const FParams& p, cudaStream_t st) {
 cudaError_t launch_fstage_pre(const FParams& p, cudaStream_t s) {
   if (p.CB <= 0) return cudaSuccess;
   switch (2 * p.nchan) {  // N = 2 nchan complex points
-    case 8: return launch_pre_L<8>(p, s);
-    case 16: return launch_pre_L<16>(p, s);
-    case 32: return launch_pre_L<32>(p, s);
-    case 64: return launch_pre_L<64>(p, s);
-    case 128: return launch_pre_L<128>(p, s);
-    case 256: return launch_pre_L<256>(p, s);
-    case 512: return launch_pre_L<512>(p, s);
-    case 1024: return launch_pre_L<1024>(p, s);
-    case 2048: return launch_pre_L<2048>(p, s);
-    case 4096: return launch_pre_L<4096>(p, s);
-    case 8192: return launch_pre_L<8192>(p, s);
-    default: return cudaErrorInvalidValue;
+    case 8: return launch_L<8>(p, s);
+    case 16: return launch_L<16>(p, s);
+    case 32: return launch_L<32>(p, s);
+    case 64: return launch_L<64>(p, s);
+    case 128: return launch_L<128>(p, s);
+    case 256: return launch_L<256>(p, s);
+    case 512: return launch_L<512>(p, s);
+    default: return launch_fstage_pre_large(p, s);
   }
 }
 
