@@ -13,8 +13,7 @@
 //
 // Operand tiles: 128 rows x 128 bytes, K-major with the 128-byte swizzle:
 // 64 blocks of FP16 or 128 blocks of E4M3 per row, written by the F step
-// (directly, or by the corner turns k_tiles / k_tiles8 from FP16 / FP8
-// spectra); the X kernel k_xmma2 streams them with bulk copies into shared
+// (directly, or by the corner turn k_tiles from FP16 / FP8 spectra); the X kernel k_xmma2 streams them with bulk copies into shared
 // memory, issues the MMAs into TMEM accumulators and adds V_ab into FP32
 // partial sums in global memory.  Both element types advance 32 bytes of a
 // row per MMA, so the shared-memory descriptors are the same.
@@ -364,25 +363,33 @@ cudaError_t launch_xtc2(const XTC2Params& p_in, int sm_count, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Corner turn of FP16 spectra into operand tiles, for FFT lengths at which
-// the F step cannot hold 8 blocks of spectra in shared memory.  One CTA takes
-// CH channels of one stream and one 64-block K tile:
-//   stage   the spectra of all stations and the tile's 64 blocks, split into
-//           Re and Im rows of 64 FP16 values (one 128-byte tile row each, in
-//           block order; rows 144 bytes apart so that neighbouring channels
-//           fall in different banks), from 16-byte reads of 4 channels, four
-//           blocks per thread;
+// Corner turn of FP16 or E4M3 spectra into operand tiles, for FFT lengths at
+// which the F step cannot hold 8 blocks of spectra in shared memory.  One CTA
+// takes CH channels of up to SB stations of one stream and one K tile (64
+// blocks of FP16, 128 of E4M3):
+//   stage   the spectra of the stations and the tile's blocks, split into Re
+//           and Im rows of 128 bytes (one tile row each, in block order; rows
+//           144 bytes apart so that neighbouring channels fall in different
+//           banks), from 16-byte reads, four blocks per thread;
 //   write   8 threads per row, one 16-byte chunk each, to the chunk's swizzled
 //           place: every tile row is written as one whole 128-byte line.
 // Blocks at or beyond cb are written as zeros (the MMA reads whole K tiles).
-constexpr int kTurnRow = 144;  // bytes per staged row (128 bytes of values + 16 bytes of padding)
+//
+// Bound by HBM (each value is read and written once) and by the latency of the
+// reads.  16 channels (E4M3: 32) make a read 64 consecutive bytes; as few stations as keep the staged rows within 74 KB let three CTAs
+// share an SM, so that one writes while the others read.  All stations of 64
+// in one CTA left room for 8 E4M3 or 4 FP16 channels, 16 bytes of each 32-byte
+// sector (64 stations x 32 streams x 4096 channels x 512 blocks of
+// E4M3: 5.46 ms, 3.98 now; 17 x 7 x 2048 x 512 of FP16: 273 and 178 us).
+constexpr int kTurnRow = 144;   // bytes per staged row (128 bytes of values + 16 bytes of padding)
+constexpr int kTurnRows = 512;  // staged rows per CTA: 2 (Re, Im) x stations x channels
+template <bool FP8> constexpr int kTurnCh = FP8 ? 32 : 16;  // channels per CTA: 64 bytes of a spectrum
 
-// Write phase of both corner turns: 8 threads per staged row, one 16-byte
-// chunk each, to the chunk's swizzled place, so every tile row is written as
-// one whole 128-byte line.
-__device__ __forceinline__ void write_staged_rows(const unsigned char* turn_raw, const TcTiles& o, int S, int nch,
-                                                  int CH, int c0, int kt, int jo) {
-  // a thread keeps one (channel, 16-byte chunk) pair and runs over the 2S
+// Write phase: stations [s0, s0 + ns).
+template <int CH>
+__device__ __forceinline__ void write_staged_rows(const unsigned char* turn_raw, const TcTiles& o, int S, int s0, int ns,
+                                                  int nch, int c0, int kt, int jo) {
+  // a thread keeps one (channel, 16-byte chunk) pair and runs over the 2 ns
   // rows (station, Re/Im) of that channel: the tile coordinates of the
   // channel are divided out once per thread, not once per chunk
   const int per = CH * 8;                  // (channel, chunk) pairs; CH * 8 divides the 256 threads
@@ -395,99 +402,51 @@ __device__ __forceinline__ void write_staged_rows(const unsigned char* turn_raw,
   const int tg = cw / o.cpt;
   const int cl = cw - tg * o.cpt;
   unsigned char* tile = o.tiles + ((((size_t)jo * o.nslice + sl) * o.NKT + kt) * 2 + tg) * 16384;
-  for (int rs = threadIdx.x / per; rs < 2 * S; rs += blockDim.x / per) {
-    const int ri = rs >= S ? 1 : 0;
-    const int s = rs - ri * S;
+  for (int rs = threadIdx.x / per; rs < 2 * ns; rs += blockDim.x / per) {
+    const int ri = rs >= ns ? 1 : 0;
+    const int s = rs - ri * ns;
     const uint4 v = *reinterpret_cast<const uint4*>(turn_raw + ((size_t)rs * CH + c) * kTurnRow + kc * 16);
-    const int r = (cl * S + s) * 2 + ri;
+    const int r = (cl * S + s0 + s) * 2 + ri;
     *reinterpret_cast<uint4*>(tile + (r >> 3) * 1024 + (r & 7) * 128 + ((kc ^ (r & 7)) << 4)) = v;
   }
 }
 
-__global__ void __launch_bounds__(256) k_tiles(const __half2* __restrict__ spec, TcTiles o, int CB, int cb, int S,
-                                               int nchan, int CH) {
-  extern __shared__ __align__(16) unsigned char turn_raw[];  // [Re/Im][S][CH] rows of kTurnRow bytes
-  const int c0 = blockIdx.x * CH;
-  const int kt = blockIdx.y;
-  const int jo = blockIdx.z;
-  const int nch = min(CH, nchan - c0);
-  const int tid = threadIdx.x;
-  // staging: a thread takes 4 channels x 4 consecutive blocks of one station
-  // (four 16-byte loads in flight), and stores per channel the 4 Re and the
-  // 4 Im values as one 8-byte piece of each row.  Threads run over blocks
-  // fastest, so a half-warp fills 64-byte runs of two rows that sit in
-  // different banks (rows 4 apart are 576 bytes apart).
-  const int lcv = CH == 16 ? 2 : (CH == 8 ? 1 : 0);  // CV = CH / 4 = 2^lcv
-  const int nstage = S * 2 * (8 << lcv);
-  // the loads of two items are issued before either item's stores, so
-  // eight 16-byte loads are in flight per thread (the kernel is bound by the
-  // latency of its HBM reads)
-  auto decode = [&](int i, int& c, int& sb, int& b0) {
-    const int b4 = i & 7;
-    const int j = i >> 3;
-    c = 4 * (j & ((1 << lcv) - 1));
-    const int rest = j >> lcv;
-    sb = rest >> 1;
-    b0 = (rest & 1) * 32 + b4 * 4;
-  };
-  for (int i0 = tid; i0 < nstage; i0 += 2 * blockDim.x) {
-    uint4 v[2][4];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = i0 + h * blockDim.x;
-      int c, sb, b0;
-      decode(i, c, sb, b0);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int bg = kt * 64 + b0 + u;
-        v[h][u] = make_uint4(0u, 0u, 0u, 0u);
-        if (i < nstage && c < nch && bg < cb)
-          v[h][u] = __ldg(reinterpret_cast<const uint4*>(spec + (((size_t)jo * CB + bg) * S + sb) * (size_t)nchan + c0 + c));
-      }
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = i0 + h * blockDim.x;
-      if (i >= nstage) break;
-      int c, sb, b0;
-      decode(i, c, sb, b0);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t w[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = e == 0 ? v[h][u].x : e == 1 ? v[h][u].y : e == 2 ? v[h][u].z : v[h][u].w;
-        const uint2 re = make_uint2((w[0] & 0xFFFFu) | (w[1] << 16), (w[2] & 0xFFFFu) | (w[3] << 16));
-        const uint2 im = make_uint2((w[0] >> 16) | (w[1] & 0xFFFF0000u), (w[2] >> 16) | (w[3] & 0xFFFF0000u));
-        *reinterpret_cast<uint2*>(turn_raw + ((size_t)sb * CH + c + e) * kTurnRow + 2 * b0) = re;
-        *reinterpret_cast<uint2*>(turn_raw + ((size_t)(S + sb) * CH + c + e) * kTurnRow + 2 * b0) = im;
-      }
-    }
-  }
-  __syncthreads();
-  write_staged_rows(turn_raw, o, S, nch, CH, c0, kt, jo);
+// 16 bytes, with their whole 128-byte line brought into L2: the CTA of the next
+// channels reads its other half.
+__device__ __forceinline__ uint4 load_line16(const void* p) {
+  uint4 v;
+  asm("ld.global.nc.L2::128B.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(p));
+  return v;
 }
 
-// FP8 corner turn: the same, for E4M3 spectra (two bytes per channel: Re,
-// Im) and 128-block K tiles.  A thread takes 8 channels (one 16-byte read) x
-// 4 consecutive blocks of one station and stores per channel 4 Re and 4 Im
-// bytes; threads run over blocks fastest, so a warp fills one whole 128-byte
-// staged row.
-__global__ void __launch_bounds__(256) k_tiles8(const uint16_t* __restrict__ spec8, TcTiles o, int CB, int cb,
-                                                int S, int nchan, int CH) {
-  extern __shared__ __align__(16) unsigned char turn_raw[];  // [Re/Im][S][CH] rows of kTurnRow bytes
+// FP16: a thread takes 4 channels (one 16-byte read) x 4 consecutive blocks of
+// one station and stores per channel the 4 Re and the 4 Im values as one
+// 8-byte piece of each row; E4M3: 8 channels, 4 Re and 4 Im bytes.  The
+// threads of one (station, block) read consecutive pieces.  The loads of two
+// items are issued before either item's stores: eight 16-byte loads in flight
+// per thread.
+template <bool FP8>
+__global__ void __launch_bounds__(256) k_tiles(const unsigned char* __restrict__ spec, TcTiles o, int CB, int cb, int S,
+                                               int nchan, int SB) {
+  constexpr int CH = kTurnCh<FP8>;
+  extern __shared__ __align__(16) unsigned char turn_raw[];  // [Re/Im][station][CH] rows of kTurnRow bytes
+  constexpr int EB = FP8 ? 2 : 4, CV = 16 / EB;   // bytes of a value, channels per read
+  constexpr int KB = FP8 ? 128 : 64, B4 = KB / 4; // blocks of the K tile, and groups of four
   const int c0 = blockIdx.x * CH;
   const int kt = blockIdx.y;
-  const int jo = blockIdx.z;
+  const int nsg = (S + SB - 1) / SB;
+  const int jo = blockIdx.z / nsg;
+  const int s0 = (blockIdx.z - jo * nsg) * SB, ns = min(SB, S - s0);
   const int nch = min(CH, nchan - c0);
   const int tid = threadIdx.x;
-  const int lcv = CH == 16 ? 1 : 0;  // CV = CH / 8 = 2^lcv
-  const int nstage = S * (32 << lcv);
-  // two items' loads before either item's stores (eight 16-byte loads in flight)
+  constexpr int cvs = CH / CV;                    // reads per (station, block)
+  const int nstage = ns * cvs * B4;
   auto decode = [&](int i, int& b4, int& c, int& sb) {
-    b4 = i & 31;
-    const int j = i >> 5;
-    c = 8 * (j & ((1 << lcv) - 1));
-    sb = j >> lcv;
+    c = CV * (i & (cvs - 1));
+    b4 = i / cvs & (B4 - 1);
+    sb = i / (cvs * B4);
   };
   for (int i0 = tid; i0 < nstage; i0 += 2 * blockDim.x) {
     uint4 v[2][4];
@@ -498,10 +457,10 @@ __global__ void __launch_bounds__(256) k_tiles8(const uint16_t* __restrict__ spe
       decode(i, b4, c, sb);
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int bg = kt * 128 + 4 * b4 + u;
+        const int bg = kt * KB + 4 * b4 + u;
         v[h][u] = make_uint4(0u, 0u, 0u, 0u);
         if (i < nstage && c < nch && bg < cb)
-          v[h][u] = __ldg(reinterpret_cast<const uint4*>(spec8 + (((size_t)jo * CB + bg) * S + sb) * (size_t)nchan + c0 + c));
+          v[h][u] = load_line16(spec + ((((size_t)jo * CB + bg) * S + s0 + sb) * (size_t)nchan + c0 + c) * EB);
       }
     }
 #pragma unroll
@@ -510,156 +469,60 @@ __global__ void __launch_bounds__(256) k_tiles8(const uint16_t* __restrict__ spe
       if (i >= nstage) break;
       int b4, c, sb;
       decode(i, b4, c, sb);
+      unsigned char* re_row = turn_raw + ((size_t)sb * CH + c) * kTurnRow;
+      unsigned char* im_row = re_row + (size_t)ns * CH * kTurnRow;
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
+      for (int e = 0; e < CV; ++e) {
         uint32_t w[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int q = e >> 1;
+          const int q = e * EB / 4;  // the value's 32-bit word
           w[u] = q == 0 ? v[h][u].x : q == 1 ? v[h][u].y : q == 2 ? v[h][u].z : v[h][u].w;
         }
-        // channel e sits in bytes 0,1 (even e) or 2,3 (odd e) of its word
-        const uint32_t sre = (e & 1) ? 0x0062u : 0x0040u, sim = (e & 1) ? 0x0073u : 0x0051u;
-        const uint32_t re = __byte_perm(__byte_perm(w[0], w[1], sre), __byte_perm(w[2], w[3], sre), 0x5410);
-        const uint32_t im = __byte_perm(__byte_perm(w[0], w[1], sim), __byte_perm(w[2], w[3], sim), 0x5410);
-        *reinterpret_cast<uint32_t*>(turn_raw + ((size_t)sb * CH + c + e) * kTurnRow + 4 * b4) = re;
-        *reinterpret_cast<uint32_t*>(turn_raw + ((size_t)(S + sb) * CH + c + e) * kTurnRow + 4 * b4) = im;
+        if constexpr (FP8) {
+          // channel e sits in bytes 0,1 (even e) or 2,3 (odd e) of its word
+          const uint32_t sre = (e & 1) ? 0x0062u : 0x0040u, sim = (e & 1) ? 0x0073u : 0x0051u;
+          *reinterpret_cast<uint32_t*>(re_row + e * kTurnRow + 4 * b4) =
+              __byte_perm(__byte_perm(w[0], w[1], sre), __byte_perm(w[2], w[3], sre), 0x5410);
+          *reinterpret_cast<uint32_t*>(im_row + e * kTurnRow + 4 * b4) =
+              __byte_perm(__byte_perm(w[0], w[1], sim), __byte_perm(w[2], w[3], sim), 0x5410);
+        } else {
+          *reinterpret_cast<uint2*>(re_row + e * kTurnRow + 8 * b4) =
+              make_uint2(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410));
+          *reinterpret_cast<uint2*>(im_row + e * kTurnRow + 8 * b4) =
+              make_uint2(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632));
+        }
       }
     }
   }
   __syncthreads();
-  write_staged_rows(turn_raw, o, S, nch, CH, c0, kt, jo);
+  write_staged_rows<CH>(turn_raw, o, S, s0, ns, nch, c0, kt, jo);
 }
 
-// Persistent FP16 corner turn: each CTA walks work items (channel group,
-// K tile, stream); item i+1's spectra are copied with cp.async into the
-// other half of a double-buffered raw stage ([station][block][CH] as 16-byte
-// pieces of 4 channels) while item i is rearranged from the raw stage into
-// the staged tile rows and written, so that the HBM reads of one item
-// overlap the rearrangement and the writes of the one before.
-__global__ void __launch_bounds__(256, 1) k_tiles_p(const __half2* __restrict__ spec, TcTiles o, int CB, int cb,
-                                                   int S, int nchan, int CH, int ngroups, int nitems) {
-  extern __shared__ __align__(16) unsigned char tp_raw[];
-  const int PPR = CH / 4;                                  // 16-byte pieces per (station, block)
-  const int raw_pieces = S * 64 * PPR;                     // per raw buffer
-  uint4* raw = reinterpret_cast<uint4*>(tp_raw);           // [2][S][64][PPR]
-  unsigned char* turn_raw = tp_raw + (size_t)2 * raw_pieces * 16;  // [Re/Im][S][CH] rows of kTurnRow bytes
-  const uint32_t raw_s = (uint32_t)__cvta_generic_to_shared(raw);
-  const int tid = threadIdx.x;
-  auto decode_item = [&](int it, int& c0, int& kt, int& jo) {
-    const int cg = it % ngroups;
-    const int rest = it / ngroups;
-    c0 = cg * CH;
-    kt = rest % o.NKT;
-    jo = rest / o.NKT;
-  };
-  auto issue = [&](int it, int buf) {
-    if (it < nitems) {
-      int c0, kt, jo;
-      decode_item(it, c0, kt, jo);
-      for (int e = tid; e < raw_pieces; e += blockDim.x) {
-        const int q = e % PPR;
-        const int row = e / PPR;                           // sb * 64 + block
-        const int blk = row & 63;
-        const int sb = row >> 6;
-        const int bg = kt * 64 + blk;
-        const int c = c0 + 4 * q;
-        const bool in = bg < cb && c < nchan;
-        const __half2* src = spec + (((size_t)jo * CB + (in ? bg : 0)) * S + sb) * (size_t)nchan + (in ? c : 0);
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(raw_s + (uint32_t)((buf * raw_pieces + e) * 16)),
-                     "l"(src), "r"(in ? 16 : 0));
-      }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  const int lcv = CH == 16 ? 2 : (CH == 8 ? 1 : 0);        // CV = CH / 4 = 2^lcv
-  const int nstage = S * 2 * (8 << lcv);
-  int buf = 0;
-  issue(blockIdx.x, 0);
-  for (int it = blockIdx.x; it < nitems; it += gridDim.x, buf ^= 1) {
-    issue(it + gridDim.x, buf ^ 1);
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    __syncthreads();  // raw[buf] has landed; the previous item's rows are written
-    int c0, kt, jo;
-    decode_item(it, c0, kt, jo);
-    const int nch = min(CH, nchan - c0);
-    const uint4* rb = raw + buf * raw_pieces;
-    for (int i = tid; i < nstage; i += blockDim.x) {
-      const int b4 = i & 7;
-      const int j = i >> 3;
-      const int c = 4 * (j & ((1 << lcv) - 1));
-      const int rest = j >> lcv;
-      const int sb = rest >> 1;
-      const int b0 = (rest & 1) * 32 + b4 * 4;
-      uint4 v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) v[u] = rb[(sb * 64 + b0 + u) * PPR + (c >> 2)];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        uint32_t w[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) w[u] = e == 0 ? v[u].x : e == 1 ? v[u].y : e == 2 ? v[u].z : v[u].w;
-        const uint2 re = make_uint2((w[0] & 0xFFFFu) | (w[1] << 16), (w[2] & 0xFFFFu) | (w[3] << 16));
-        const uint2 im = make_uint2((w[0] >> 16) | (w[1] & 0xFFFF0000u), (w[2] >> 16) | (w[3] & 0xFFFF0000u));
-        *reinterpret_cast<uint2*>(turn_raw + ((size_t)sb * CH + c + e) * kTurnRow + 2 * b0) = re;
-        *reinterpret_cast<uint2*>(turn_raw + ((size_t)(S + sb) * CH + c + e) * kTurnRow + 2 * b0) = im;
-      }
-    }
-    __syncthreads();
-    // the rows of this item's channels; threads of channels beyond nch skip
-    // the writes (no barrier inside)
-    write_staged_rows(turn_raw, o, S, nch, CH, c0, kt, jo);
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
+template <bool FP8>
+static cudaError_t launch_turn(const void* spec, const TcTiles& o, int CB, int cb, int S, int G, int nchan, cudaStream_t s) {
+  if (cb <= 0) return cudaSuccess;
+  constexpr int CH = kTurnCh<FP8>;
+  if (nchan % (FP8 ? 8 : 4)) return cudaErrorInvalidValue;
+  // stations per CTA: equal shares of at most kTurnRows rows
+  const int groups = (2 * S * CH + kTurnRows - 1) / kTurnRows;
+  const int SB = (S + groups - 1) / groups;
+  const size_t smem = (size_t)2 * SB * CH * kTurnRow;
+  cudaError_t e = cudaFuncSetAttribute(k_tiles<FP8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const dim3 grid((nchan + CH - 1) / CH, o.NKT, G * ((S + SB - 1) / SB));
+  k_tiles<FP8><<<grid, 256, smem, s>>>(static_cast<const unsigned char*>(spec), o, CB, cb, S, nchan, SB);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_tiles(const __half2* spec, const TcTiles& o, int CB, int cb, int S, int G, int nchan,
                          cudaStream_t s) {
-  if (cb <= 0) return cudaSuccess;
-  {
-    // persistent form: raw double buffer + staged rows = 800 S CH bytes <= 210 KB
-    int CH = 16;
-    while (CH > 4 && (size_t)800 * S * CH > 210 * 1024) CH /= 2;
-    const size_t smem = (size_t)800 * S * CH;
-    if (smem <= 210 * 1024 && nchan >= 4) {
-      static int sm_count = 0;
-      if (!sm_count) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-          sm_count = 152;
-      }
-      const int ngroups = (nchan + CH - 1) / CH;
-      const int nitems = ngroups * o.NKT * G;
-      cudaError_t e = cudaFuncSetAttribute(k_tiles_p, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-      k_tiles_p<<<std::min(nitems, sm_count), 256, smem, s>>>(spec, o, CB, cb, S, nchan, CH, ngroups, nitems);
-      return cudaGetLastError();
-    }
-  }
-  // channels per CTA: the staged rows stay within about 100 KB
-  int CH = 16;
-  while (CH > 4 && (size_t)2 * S * CH * kTurnRow > 100 * 1024) CH /= 2;
-  const size_t smem = (size_t)2 * S * CH * kTurnRow;
-  cudaError_t e = cudaFuncSetAttribute(k_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((nchan + CH - 1) / CH, o.NKT, G);
-  k_tiles<<<grid, 256, smem, s>>>(spec, o, CB, cb, S, nchan, CH);
-  return cudaGetLastError();
+  return launch_turn<false>(spec, o, CB, cb, S, G, nchan, s);
 }
 
 cudaError_t launch_tiles8(const uint16_t* spec8, const TcTiles& o, int CB, int cb, int S, int G, int nchan,
                           cudaStream_t s) {
-  if (cb <= 0) return cudaSuccess;
-  if (nchan % 8) return cudaErrorInvalidValue;
-  int CH = 16;
-  while (CH > 8 && (size_t)2 * S * CH * kTurnRow > 110 * 1024) CH /= 2;
-  const size_t smem = (size_t)2 * S * CH * kTurnRow;
-  cudaError_t e = cudaFuncSetAttribute(k_tiles8, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid((nchan + CH - 1) / CH, o.NKT, G);
-  k_tiles8<<<grid, 256, smem, s>>>(spec8, o, CB, cb, S, nchan, CH);
-  return cudaGetLastError();
+  return launch_turn<true>(spec8, o, CB, cb, S, G, nchan, s);
 }
 
 int xtc_cpt(int S) { return S <= 64 ? 64 / S : 0; }
