@@ -672,7 +672,7 @@ static FParams fparams(corr_t* h, int blk0, int cb, int slot) {
 }
 
 // Device work of one integration after its delay blocks are in descriptor
-// slot `slot`: partial-sum clear, F and X per chunk, weights and
+// slot `slot`: F and X per chunk, weights and
 // normalisation, with no host wait (so it can be recorded into a CUDA graph).
 // M = blocks of the integration.  With `overlap` the X step of each chunk
 // runs on xstream while the F step of the next chunk runs on st (two
@@ -680,6 +680,7 @@ static FParams fparams(corr_t* h, int blk0, int cb, int slot) {
 // before the weights.  Without it every launch goes to st.
 static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, double* w_out, int slot, bool overlap) {
   const int S = h->S;
+  overlap = overlap && M > h->CB;  // a single chunk has nothing to overlap with: no second stream, no events
   cudaEvent_t pa = nullptr;
   const bool reduced = h->precision != CORR_PREC_FP32;  // FP16 / FP8 spectra
   const bool fp8 = h->precision == CORR_PREC_FP8_TC;
@@ -688,12 +689,18 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
   // the X step's stations and streams (2S and nsub with both hands)
   const int XS = x_stations(h), XG = x_streams(h);
   cudaStream_t xs = overlap ? h->xstream : st;
-  CK(cudaMemsetAsync(h->d_part, 0, sizeof(float2) * (size_t)kz_used * nbl_of(XS) * XG * h->nchan, st),
-     "partials memset");
+  // chunks of equal length (in whole K tiles on the tensor cores), as few as
+  // the buffers allow: a short last one would leave most SMs idle (64 blocks
+  // after 19 chunks of 819 cost the time of 120)
+  int step = h->CB;
+  if (h->chunk_req <= 0) {
+    const int n = (M + h->CB - 1) / h->CB, kb = tc ? (fp8 ? 128 : 64) : 1;
+    step = std::min(h->CB, ((M + n - 1) / n + kb - 1) / kb * kb);
+  }
   int c = 0;
-  for (int c0 = 0; c0 < M; c0 += h->CB, ++c) {
+  for (int c0 = 0; c0 < M; c0 += step, ++c) {
     const int buf = overlap ? (c & 1) : 0;
-    const int cb = (M - c0 < h->CB) ? (M - c0) : h->CB;
+    const int cb = (M - c0 < step) ? (M - c0) : step;
     // the F step writes buffer `buf`: the X step that read it last must be done
     if (overlap && h->x_pending[buf]) {
       CK(cudaStreamWaitEvent(st, h->ev_x[buf], 0), "wait for the X step");
@@ -744,6 +751,7 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
       xp.W = o.W;
       xp.fp8 = o.fp8;
       xp.part = h->d_part;
+      xp.first = c0 == 0;
       xp.err = h->d_err;
       pa = prof_begin(h, xs);
       CK(launch_xtc2(xp, h->sm_count, xs), "tensor-core xstage launch");
@@ -765,6 +773,7 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
       xp.nchan = h->nchan;
       xp.KZ = h->KZ;
       xp.part = h->d_part;
+      xp.first = c0 == 0;
       xp.err = h->d_err;
       pa = prof_begin(h, xs);
       CK(launch_xstage(xp, xs), "xstage launch");

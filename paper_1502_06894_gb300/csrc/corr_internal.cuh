@@ -103,6 +103,7 @@ struct XTC2Params {
   int nslice, NKT, S, G, nchan, cpt, W;
   int fp8;                  // tiles hold E4M3 values (MMA kind::f8f6f4) instead of FP16 (kind::f16)
   float2* part;             // [G][nchan][nbl]
+  int first;                // 1: write the partial sums (the integration's first chunk) instead of adding to them
   int* err;
   long long wait_limit;     // spins per mbarrier wait (set by the launcher)
 };
@@ -114,6 +115,7 @@ struct XParams {
   int CB, S, G, nchan;
   int KZ;                   // block splits per chunk (one partial each)
   float2* part;             // [KZ][nbl][G][nchan]
+  int first = 0;            // 1: write the partial sums (the integration's first chunk) instead of adding to them
   int* err;                 // set to 1 when a device wait times out (may be null)
   long long wait_limit;     // spins per mbarrier wait (set by the launcher)
 };

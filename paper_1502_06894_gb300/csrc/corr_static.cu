@@ -185,9 +185,7 @@ extern "C" int corr_correlate_static(const corr_scan_desc* d, int64_t integratio
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(base + o_c, d->seg_coeffs, sizeof(double) * S * kMaxSegs * 6, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(base + o_nu0, d->nu0_hz, sizeof(double) * nsub, cudaMemcpyHostToDevice, st);
-  // the X partial sums accumulate and the timeout flag latches, so both start
-  // at zero on every call
-  if (e == cudaSuccess) e = cudaMemsetAsync(base + o_part, 0, per_part * KZ, st);
+  // the timeout flag latches, so it starts at zero on every call
   if (e == cudaSuccess) e = cudaMemsetAsync(base + o_err, 0, sizeof(int), st);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -255,6 +253,7 @@ extern "C" int corr_correlate_static(const corr_scan_desc* d, int64_t integratio
     xp.nchan = nchan;
     xp.KZ = KZ;
     xp.part = (float2*)(base + o_part);
+    xp.first = c0 == 0;
     xp.err = (int*)(base + o_err);
     e = launch_xstage(xp, st);
   }

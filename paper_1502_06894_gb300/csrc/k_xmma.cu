@@ -320,9 +320,12 @@ __global__ void __launch_bounds__(160, 1) k_xmma2(XTC2Params p, int nitems) {
       const int nf = nch * nbl * 2;  // a multiple of 4: nch is even
       for (int e = 4 * r; e < nf; e += 4 * 128) {
         const float4 x = *reinterpret_cast<const float4*>(src + e);
-        asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x.x), "f"(x.y), "f"(x.z),
-                     "f"(x.w)
-                     : "memory");
+        if (p.first)
+          *reinterpret_cast<float4*>(dst + e) = x;
+        else
+          asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e), "f"(x.x), "f"(x.y), "f"(x.z),
+                       "f"(x.w)
+                       : "memory");
       }
       asm volatile("bar.sync 1, 128;" ::: "memory");  // stage free for the next item
     }

@@ -168,16 +168,20 @@ __device__ __forceinline__ void tile_block(float2 (&acc)[TS][TS], const unsigned
 }
 
 // Add a tile pair's sums to the partial sums: part[baseline * row] of this
-// lane's stream and channel, one add per element and launch.
+// lane's stream and channel, one add per element and launch (the first
+// launch of an integration writes them, so that nothing clears them before).
 template <int TS, bool DIAG>
-__device__ __forceinline__ void add_tile(const float2 (&acc)[TS][TS], float2* part, size_t row, int a0, int b0, int S) {
+__device__ __forceinline__ void add_tile(const float2 (&acc)[TS][TS], float2* part, size_t row, int a0, int b0, int S,
+                                         int first) {
 #pragma unroll
   for (int i = 0; i < TS; ++i)
 #pragma unroll
     for (int j = DIAG ? i : 0; j < TS; ++j)
       if (a0 + i < S && b0 + j < S) {
         float2* dst = part + (size_t)bl_index(a0 + i, b0 + j, S) * row;
-        if (DIAG && j == i)
+        if (first)
+          *dst = DIAG && j == i ? auto_value(acc[i][j]) : acc[i][j];
+        else if (DIAG && j == i)
           atomicAdd(&dst->x, auto_value(acc[i][j]).x);
         else
           asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(dst), "f"(acc[i][j].x), "f"(acc[i][j].y) : "memory");
@@ -224,7 +228,7 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
   const int g = blockIdx.y, kz = blockIdx.z;
   const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
   const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
-  if (b_hi <= b_lo) return;
+  if (b_hi <= b_lo && !p.first) return;  // an empty range of the first chunk writes zeros
   const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
   const int row_bytes = sh.pitch * EB;
   Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
@@ -275,7 +279,8 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
   }
   if (k < p.nchan) {
     const size_t row = (size_t)p.G * p.nchan;
-    add_tile<TS, true>(acc, p.part + (size_t)kz * nbl_of(TS) * row + (size_t)g * p.nchan + k, row, 0, 0, TS);
+    add_tile<TS, true>(acc, p.part + (size_t)kz * nbl_of(TS) * row + (size_t)g * p.nchan + k, row, 0, 0, TS,
+                       p.first);
   }
   __syncthreads();
   if (s_abort && threadIdx.x == 0) ring.drain(p.err);
@@ -311,7 +316,7 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
   const int g = blockIdx.y, kz = blockIdx.z, S = p.S;
   const int b_lo = (int)((int64_t)p.CB * kz / p.KZ);
   const int b_hi = (int)((int64_t)p.CB * (kz + 1) / p.KZ);
-  if (b_hi <= b_lo) return;
+  if (b_hi <= b_lo && !p.first) return;  // an empty range of the first chunk writes zeros
   const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
   const int row_bytes = sh.pitch * 8, nwarp = gr.nwarp;
   Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
@@ -367,7 +372,7 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
     if (k0 + lane < p.nchan) {
       const size_t row = (size_t)p.G * p.nchan;
       add_tile<TS, DIAG>(acc, p.part + (size_t)kz * nbl_of(S) * row + (size_t)g * p.nchan + k0 + lane, row,
-                         gr.tile[wa] * TS, gr.tile[wb] * TS, S);
+                         gr.tile[wa] * TS, gr.tile[wb] * TS, S, p.first);
     }
   };
   if (warp < nwarp) {  // a CTA with fewer pairs than the largest one has warps without work
