@@ -1136,11 +1136,16 @@ static cudaError_t launch_LG(const FParams& p, cudaStream_t st) {
   const int base = std::max(1, std::min(64, NGRP / p.G));
   // Codes turned stream by stream: the turned codes of all streams (of 16 at a
   // time if more do not fit) beside the windows, as long as they cost no CTA
-  // per SM; two blocks at a time where they fit too (a step ends at a barrier).
+  // per SM.  A step ends at barriers, so it takes four rounds of transforms if
+  // the windows fit and two waves of CTAs stay (1024 samples, 8, 16, 32
+  // streams, which two blocks make 1, 2 and 4 rounds: 422, 353, 318 us).
   if constexpr (Codes<L, PRE>::on) {
     const int most = std::max(1, resident(kWordsOffset<L>(NGRP) + window(base)));
-    if (base == 1 && resident(turned(2, p.G)) >= most && p.CB >= 2)
-      return launch_turn<L, GC, PRE, true>(p, 2, wslot, p.G, steps_per_cta(2, most), turned(2, p.G), st);
+    const int64_t keep = (int64_t)p.CB * p.S / ((int64_t)2 * most * sm_count);  // blocks a CTA, for two waves
+    int slots = (int)std::min<int64_t>(std::min(64, (4 * NGRP + p.G - 1) / p.G), std::max<int64_t>(base, keep));
+    while (slots > base && resident(turned(slots, p.G)) < most) --slots;
+    if (slots > base)
+      return launch_turn<L, GC, PRE, true>(p, slots, wslot, p.G, steps_per_cta(slots, most), turned(slots, p.G), st);
     for (const int jb : {p.G, 16})
       if (jb <= p.G && resident(turned(base, jb)) >= most)
         return launch_turn<L, GC, PRE, true>(p, base, wslot, jb, steps_per_cta(base, most), turned(base, jb), st);
