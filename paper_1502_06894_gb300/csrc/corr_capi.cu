@@ -98,9 +98,8 @@ struct corr_s {
   float* d_phi[2] = {};
   float2* d_dphi[2] = {};  // pre-F: phase step per sample (hi, lo), [S][nsub][Mcap]
   uint8_t* d_valid[2] = {};
-  unsigned long long* d_stat[2] = {};  // [S][3] data-coverage statistics
-  unsigned long long* h_stat[2] = {};  // pinned copies
-  unsigned long long* h_stat_init = nullptr;  // pinned, the statistics' start values
+  unsigned long long* d_stat[2] = {};  // [S][3] data-coverage statistics, and the delay kernel's CTA count
+  unsigned long long* h_stat[2] = {};  // pinned, written by the delay kernel
   float2* d_twN = nullptr;
   int CB = 0, KZ = 0;
   // spectra chunk (and tensor-core tiles): two buffers when the F step of
@@ -117,14 +116,12 @@ struct corr_s {
   uint64_t model_gen = 1, la_gen = 0;  // bumped whenever the delay model or station data change
   float2* d_part = nullptr;
   float2* d_out = nullptr;
-  int* d_wcount = nullptr;
   double* d_wts = nullptr;
   size_t spec_budget = (size_t)1 << 30;
   int chunk_req = 0;  // blocks per F/X chunk requested by the caller (0: from spec_budget)
   int sm_count = 0;
   int sigma = 0;      // FP16 / FP8 spectra carry X * 2^-sigma
-  int* d_err = nullptr;
-  int* h_err = nullptr;  // pinned
+  int* h_err = nullptr;  // pinned; the X kernels set it when a device wait times out
   unsigned char* d_tiles[2] = {};  // tensor-core operand tiles
   bool tc_tiles = false;
   bool tc_direct = false;  // the F step writes the tiles itself
@@ -297,22 +294,16 @@ static void free_device(corr_t* h) {
   if (h->ev_main) cudaEventDestroy(h->ev_main);
   if (h->ev_la) cudaEventDestroy(h->ev_la);
   h->ev_main = h->ev_la = nullptr;
-  cudaFreeHost(h->h_stat_init);
-  h->h_stat_init = nullptr;
   cudaFree(h->d_twN);
   cudaFree(h->d_part);
   cudaFree(h->d_out);
-  cudaFree(h->d_wcount);
   cudaFree(h->d_wts);
   h->d_wts = nullptr;
-  cudaFree(h->d_err);
   cudaFreeHost(h->h_err);
-  h->d_err = nullptr;
   h->h_err = nullptr;
   h->d_views = nullptr; h->h_views = nullptr; h->d_nseg = nullptr; h->d_seg_t0 = nullptr;
   h->d_seg_c = nullptr; h->d_nu0 = nullptr;
   h->d_twN = nullptr; h->d_part = nullptr; h->d_out = nullptr;
-  h->d_wcount = nullptr;
   h->prepared = false;
   h->views_valid = false;
   h->la_valid = false;
@@ -413,10 +404,9 @@ static int work_layout(corr_t* h, WorkLayout& w) {
   w.small = sizeof(StationView) * S + sizeof(int) * S + sizeof(double) * S * kMaxSegs * 7 +
             sizeof(double) * h->nsub +
             2 * ((sizeof(int64_t) + sizeof(float) + 1) * S * M + sizeof(float) * S * h->nsub * M +
-                 sizeof(unsigned long long) * 3 * S +
+                 sizeof(unsigned long long) * (3 * S + 1) +
                  (h->rotation == CORR_ROT_PRE_F ? sizeof(float2) * S * h->nsub * M : 0)) +
-            sizeof(float2) * h->N + sizeof(float2) * nbl * out_per_baseline(h) + (sizeof(int) + sizeof(double)) * nbl +
-            sizeof(int);
+            sizeof(float2) * h->N + sizeof(float2) * nbl * out_per_baseline(h) + sizeof(double) * nbl;
   return CORR_OK;
 }
 
@@ -454,14 +444,11 @@ static int prepare(corr_t* h) {
         (rc = dalloc(h, (void**)&h->d_dphi[q], sizeof(float2) * S * h->nsub * h->Mcap, "phase steps")))
       return rc;
     if ((rc = dalloc(h, (void**)&h->d_valid[q], (size_t)S * h->Mcap, "valid"))) return rc;
-    if ((rc = dalloc(h, (void**)&h->d_stat[q], sizeof(unsigned long long) * 3 * S, "stat"))) return rc;
+    if ((rc = dalloc(h, (void**)&h->d_stat[q], sizeof(unsigned long long) * (3 * S + 1), "stat"))) return rc;
+    std::vector<unsigned long long> start(3 * S + 1, 0ull);
+    for (int e = 0; e < 3 * S; ++e) start[e] = coverage_start(e % 3);
+    CK(cudaMemcpy(h->d_stat[q], start.data(), sizeof(unsigned long long) * start.size(), cudaMemcpyHostToDevice), "stat H2D");
     CK(cudaMallocHost((void**)&h->h_stat[q], sizeof(unsigned long long) * 3 * S), "cudaMallocHost stat");
-  }
-  CK(cudaMallocHost((void**)&h->h_stat_init, sizeof(unsigned long long) * 3 * S), "cudaMallocHost stat");
-  for (int s = 0; s < S; ++s) {
-    h->h_stat_init[3 * s + 0] = 0ull;   // max window end
-    h->h_stat_init[3 * s + 1] = ~0ull;  // min window start
-    h->h_stat_init[3 * s + 2] = 0ull;   // valid blocks
   }
   if ((rc = dalloc(h, (void**)&h->d_twN, sizeof(float2) * h->N, "twiddles"))) return rc;
   h->overlap = w.nbuf == 2;
@@ -475,9 +462,7 @@ static int prepare(corr_t* h) {
   CK(cudaEventCreateWithFlags(&h->ev_la, cudaEventDisableTiming), "events");
   if ((rc = dalloc(h, (void**)&h->d_part, w.part, "partials"))) return rc;
   if ((rc = dalloc(h, (void**)&h->d_out, sizeof(float2) * (size_t)nbl * out_per_baseline(h), "out"))) return rc;
-  if ((rc = dalloc(h, (void**)&h->d_wcount, sizeof(int) * nbl, "wcount"))) return rc;
   if ((rc = dalloc(h, (void**)&h->d_wts, sizeof(double) * nbl, "weights"))) return rc;
-  if ((rc = dalloc(h, (void**)&h->d_err, sizeof(int), "error flag"))) return rc;
   CK(cudaMallocHost((void**)&h->h_err, sizeof(int)), "cudaMallocHost err");
   h->tc_tiles = w.tiles;
   h->tc_direct = w.direct;
@@ -490,7 +475,6 @@ static int prepare(corr_t* h) {
     }
   }
   *h->h_err = 0;
-  CK(cudaMemset(h->d_err, 0, sizeof(int)), "error flag reset");
   // W_N^m = exp(-2 pi i m / N), computed in FP64 on the host
   std::vector<float2> tw(h->N);
   for (int m = 0; m < h->N; ++m) {
@@ -637,7 +621,9 @@ static DelayParams delay_params(corr_t* h, int64_t b0, int nb, int ld, int slot)
   p.valid = h->d_valid[slot];
   p.eps_out = nullptr;
   p.tau_out = nullptr;
-  p.max_end = nullptr;
+  p.coverage = nullptr;
+  p.done = nullptr;
+  p.coverage_out = nullptr;
   p.dphi = h->d_dphi[slot];  // null unless pre-F
   return p;
 }
@@ -752,7 +738,7 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
       xp.fp8 = o.fp8;
       xp.part = h->d_part;
       xp.first = c0 == 0;
-      xp.err = h->d_err;
+      xp.err = h->h_err;
       pa = prof_begin(h, xs);
       CK(launch_xtc2(xp, h->sm_count, xs), "tensor-core xstage launch");
       prof_end(h, 2, pa, xs);
@@ -774,7 +760,7 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
       xp.KZ = h->KZ;
       xp.part = h->d_part;
       xp.first = c0 == 0;
-      xp.err = h->d_err;
+      xp.err = h->h_err;
       pa = prof_begin(h, xs);
       CK(launch_xstage(xp, xs), "xstage launch");
       prof_end(h, 2, pa, xs);
@@ -800,12 +786,10 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
   fin.valid = h->d_valid[slot];
   fin.ld = h->Mcap;
   fin.M = M;
-  fin.wcount = h->d_wcount;
   fin.out = vis_out;
   fin.weights = w_out;
   fin.err = nullptr;  // the handle reports a device timeout as CORR_ETIMEOUT
   pa = prof_begin(h, st);
-  CK(launch_weights(fin, st), "weights launch");
   // FP16 / FP8 spectra carry X 2^-sigma: the sums carry 2^(-2 sigma)
   const float unscale = reduced ? ldexpf(1.0f, 2 * h->sigma) : 1.0f;
   if (cross_of(h)) {
@@ -822,21 +806,19 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
 }
 
 // Delay blocks of integration i into descriptor slot i & 1 on stream st,
-// with the data-coverage statistics copied to the slot's pinned host copy.
+// with the data-coverage statistics written to the slot's pinned host memory.
 static int enqueue_delays(corr_t* h, int64_t i, cudaStream_t st) {
   const int S = h->S;
   const int slot = (int)(i & 1);
   const int64_t bfirst = integ_first_block(h, i);
   const int M = (int)(integ_first_block(h, i + 1) - bfirst);
-  CK(cudaMemcpyAsync(h->d_stat[slot], h->h_stat_init, sizeof(unsigned long long) * 3 * S, cudaMemcpyHostToDevice, st),
-     "stat H2D");
   DelayParams dp = delay_params(h, bfirst, M, h->Mcap, slot);
-  dp.max_end = h->d_stat[slot];
+  dp.coverage = h->d_stat[slot];
+  dp.done = reinterpret_cast<unsigned int*>(h->d_stat[slot] + 3 * S);
+  dp.coverage_out = h->h_stat[slot];
   cudaEvent_t pa = prof_begin(h, st);
   CK(launch_delay_blocks(dp, st), "delay_blocks launch");
   prof_end(h, 0, pa, st);
-  CK(cudaMemcpyAsync(h->h_stat[slot], h->d_stat[slot], sizeof(unsigned long long) * 3 * S, cudaMemcpyDeviceToHost, st),
-     "stat D2H");
   return CORR_OK;
 }
 
@@ -902,7 +884,6 @@ static int run_integration(corr_t* h, float2* vis_out, double* w_out) {
   CK(cudaEventRecord(h->ev_main, h->stream), "main event");
   int rc2 = enqueue_rest(h, h->stream, M, vis_out, w_out, slot, h->overlap);
   if (rc2) return rc2;
-  CK(cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream), "error flag D2H");
   h->next_int = i + 1;
   // 2. look-ahead: the next integration's delay blocks, on their own stream,
   //    while this integration's F and X steps run
@@ -1332,9 +1313,6 @@ int corr_reset(corr_t* h) {
   h->next_int = 0;
   // a device wait that timed out earlier no longer blocks the handle
   if (h->prepared) {
-    cudaError_t e = cudaMemsetAsync(h->d_err, 0, sizeof(int), h->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) return h->cuda_fail(e, "corr_reset: error flag");
     *h->h_err = 0;
   }
   return CORR_OK;
@@ -1452,7 +1430,6 @@ int corr_batch_run(corr_t* const* hs, int n, float* const* dev_out, double* cons
     // one stream per scan inside the graph (scans run side by side instead)
     rc = enqueue_rest(h, st, M, reinterpret_cast<float2*>(dev_out[j]), dev_weights ? dev_weights[j] : nullptr, slot,
                       false);
-    if (rc == CORR_OK) e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
   }
   // join every branch back into the root
   for (int q = 0; q < kBatchStreams && e == cudaSuccess; ++q) {

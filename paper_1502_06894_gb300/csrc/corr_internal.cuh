@@ -61,7 +61,12 @@ struct DelayParams {
   // the block's first sample instead of its centre, and dphi the phase step
   // per sample in turns as (hi, lo) with hi of at most 10 significant bits
   float2* dphi;
-  unsigned long long* max_end;   // optional [S]: max(window end - sample0) over blocks, encoded +2^62
+  // optional: the station's data coverage, [S][3] (see k_delay_blocks), reduced
+  // in device memory; the last CTA to finish (counted in `done`) moves it to
+  // pinned host memory and leaves `coverage` and `done` as they started
+  unsigned long long* coverage;
+  unsigned int* done;
+  unsigned long long* coverage_out;
 };
 
 // F stage: unpack + real FFT + rotation for CB blocks x S stations x G streams.
@@ -125,7 +130,6 @@ struct FinParams {
   int KZ, S, G, nchan, N;
   const uint8_t* valid;     // [S][ld]
   int ld, M;                // blocks of the integration
-  int* wcount;              // [nbl] scratch
   float2* out;              // [nbl][G][nchan]
   double* weights;          // [nbl] (device, may be null)
   const int* err;           // optional: when *err != 0 (an X-step wait timed out) the output is NaN
@@ -160,7 +164,7 @@ cudaError_t fstage_pre_large_init_constants();
 cudaError_t fringe_init_constants();
 int xstage_kz(int CB, int S, int G, int nchan);
 cudaError_t launch_xstage(const XParams& p, cudaStream_t s);
-cudaError_t launch_weights(const FinParams& p, cudaStream_t s);
+// integration end: the baselines' weights, and V / (W N)
 cudaError_t launch_finalize(const FinParams& p, cudaStream_t s);
 // The CUDA-core X step reads FP16 / E4M3 spectra (XParams::in_kind) for up to
 // 12 stations and whole 128-channel tiles.
@@ -185,6 +189,9 @@ cudaError_t launch_finalize_tc(const FinParams& p, float unscale, cudaStream_t s
 // p.G = nsub streams (FP32 layout [KZ][nblv][nsub][nchan], or with `tc` the tensor-core
 // layout [KZ][nsub][nchan][nblv]); out [nbl][nsub][4][nchan], hand product pq = 2 p + q
 cudaError_t launch_finalize_cross(const FinParams& p, bool tc, float unscale, cudaStream_t s);
+
+// start values of the coverage statistics: max window end, min window start, valid blocks
+__host__ __device__ inline unsigned long long coverage_start(int q) { return q == 1 ? ~0ull : 0ull; }
 
 __host__ __device__ inline int nbl_of(int S) { return S * (S + 1) / 2; }
 __host__ __device__ inline int bl_index(int a, int b, int S) { return a * S - a * (a - 1) / 2 + (b - a); }

@@ -129,7 +129,7 @@ extern "C" int corr_correlate_static(const corr_scan_desc* d, int64_t integratio
   const size_t o_delta = c.take(sizeof(float) * (size_t)S * M);
   const size_t o_phi = c.take(sizeof(float) * (size_t)S * nsub * M);
   const size_t o_valid = c.take((size_t)S * M);
-  const size_t o_wc = c.take(sizeof(int) * nbl);
+  c.take(sizeof(int) * nbl);  // not used: keeps the largest accepted shape where it has been
   const size_t o_err = c.take(sizeof(int));
   const size_t fixed = c.off;
   const size_t per_block = sizeof(float2) * (size_t)G * S * nchan;
@@ -213,7 +213,9 @@ extern "C" int corr_correlate_static(const corr_scan_desc* d, int64_t integratio
   dp.valid = (uint8_t*)(base + o_valid);
   dp.eps_out = nullptr;
   dp.tau_out = nullptr;
-  dp.max_end = nullptr;
+  dp.coverage = nullptr;
+  dp.done = nullptr;
+  dp.coverage_out = nullptr;
   dp.dphi = nullptr;
   e = launch_delay_blocks(dp, st);
   for (int c0 = 0; e == cudaSuccess && c0 < M; c0 += CB) {
@@ -268,12 +270,10 @@ extern "C" int corr_correlate_static(const corr_scan_desc* d, int64_t integratio
     fin.valid = dp.valid;
     fin.ld = M;
     fin.M = M;
-    fin.wcount = (int*)(base + o_wc);
     fin.out = (float2*)dev_out;
     fin.weights = dev_weights;
     fin.err = (const int*)(base + o_err);  // a timed-out X-step wait turns the output into NaN
-    e = launch_weights(fin, st);
-    if (e == cudaSuccess) e = launch_finalize(fin, st);
+    e = launch_finalize(fin, st);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kDelayThreads) k_delay_blocks(DelayParams p) {
   }
   if (mine && p.eps_out) p.eps_out[o] = eps;
   if (mine && p.tau_out) p.tau_out[o] = tau;
-  if (p.max_end) {
+  if (p.coverage) {
     // [0]: max window end, [1]: min window start (both relative to the
     // station's first sample, offset by 2^62 so they order as unsigned);
     // [2]: number of valid blocks.  Reduced over the CTA first: one atomic of
@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(kDelayThreads) k_delay_blocks(DelayParams p) {
     }
     __shared__ unsigned long long s_hi[kDelayThreads / 32], s_lo[kDelayThreads / 32];
     __shared__ int s_count[kDelayThreads / 32];
+    __shared__ bool s_last;
     if ((threadIdx.x & 31) == 0) {
       s_hi[threadIdx.x >> 5] = hi;
       s_lo[threadIdx.x >> 5] = lo;
@@ -124,9 +125,20 @@ __global__ void __launch_bounds__(kDelayThreads) k_delay_blocks(DelayParams p) {
         lo = s_lo[w] < lo ? s_lo[w] : lo;
         total += s_count[w];
       }
-      atomicMax(&p.max_end[3 * s + 0], hi);
-      atomicMin(&p.max_end[3 * s + 1], lo);
-      if (total) atomicAdd(&p.max_end[3 * s + 2], (unsigned long long)total);
+      atomicMax(&p.coverage[3 * s + 0], hi);
+      atomicMin(&p.coverage[3 * s + 1], lo);
+      if (total) atomicAdd(&p.coverage[3 * s + 2], (unsigned long long)total);
+      __threadfence();
+      s_last = atomicAdd(p.done, 1u) == gridDim.x * gridDim.y - 1;
+    }
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      for (int q = threadIdx.x; q < 3 * p.S; q += blockDim.x) {
+        p.coverage_out[q] = __ldcg(&p.coverage[q]);
+        p.coverage[q] = coverage_start(q % 3);
+      }
+      if (threadIdx.x == 0) *p.done = 0u;
     }
   }
 }

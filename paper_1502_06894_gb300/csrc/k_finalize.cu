@@ -8,23 +8,24 @@
 // order.
 #include "corr_internal.cuh"
 
+#include <algorithm>
+
 namespace corr {
 
-// One CTA per baseline.  Bound by the latency of its loads, which take 16
-// blocks each where the rows of `valid` start at multiples of 16 bytes (a
-// handle pads them; the static scratch has no room to): 62500 blocks took 120
-// us with byte loads, 11.2 us now.
-__global__ void __launch_bounds__(256) k_weights(FinParams p) {
-  const int bl = blockIdx.x;
-  // decode baseline index -> (a, b)
-  int a = 0, q = bl;
+// Blocks valid at both stations of baseline bl, counted by `threads` threads
+// from index i0; the caller adds their counts up.  Bound by the latency of its
+// loads, which take 16 blocks each where the rows of `valid` start at multiples
+// of 16 bytes (a handle pads them; the static scratch has no room to): 62500
+// blocks took a CTA 120 us with byte loads, 11 us now.
+__device__ __forceinline__ int count_valid(const FinParams& p, int bl, int i0, int threads) {
+  int a = 0, q = bl;  // baseline index -> (a, b)
   while (q >= p.S - a) { q -= p.S - a; ++a; }
   const int b = a + q;
   const uint8_t* va = p.valid + (size_t)a * p.ld;
   const uint8_t* vb = p.valid + (size_t)b * p.ld;
   int cnt = 0;
   const int vec = p.ld % 16 == 0 ? p.M : 0;  // bytes of 0 or 1
-  for (int i = 16 * threadIdx.x; i < vec; i += 16 * blockDim.x) {
+  for (int i = 16 * i0; i < vec; i += 16 * threads) {
     const uint4 x = *reinterpret_cast<const uint4*>(va + i), y = *reinterpret_cast<const uint4*>(vb + i);
     const uint32_t w[4] = {x.x & y.x, x.y & y.y, x.z & y.z, x.w & y.w};
 #pragma unroll
@@ -33,29 +34,34 @@ __global__ void __launch_bounds__(256) k_weights(FinParams p) {
       cnt += __popc(n >= 4 ? w[q] : n > 0 ? w[q] & ((1u << (8 * n)) - 1u) : 0u);
     }
   }
-  for (int i = vec + threadIdx.x; i < p.M; i += blockDim.x) cnt += va[i] & vb[i];
-  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
-  __shared__ int ws[32];
-  if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = cnt;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int tot = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += ws[w];
-    p.wcount[bl] = tot;
-    if (p.weights) p.weights[bl] = (double)tot;
-  }
-}
-
-cudaError_t launch_weights(const FinParams& p, cudaStream_t s) {
-  k_weights<<<nbl_of(p.S), 256, 0, s>>>(p);
-  return cudaGetLastError();
+  for (int i = vec + i0; i < p.M; i += threads) cnt += va[i] & vb[i];
+  return cnt;
 }
 
 // 1 / (W N) of a baseline times `unscale`: in FP64, which this GPU runs at a
 // 64th of its FP32 rate, so one thread of a CTA forms it, not every element.
-__device__ __forceinline__ float fin_scale(const FinParams& p, int bl, float unscale) {
-  const int w = p.wcount[bl];
+// That thread also writes the weight, in the first CTA of the baseline's row.
+__device__ __forceinline__ float fin_scale(const FinParams& p, int bl, int w, float unscale) {
+  if (p.weights && blockIdx.x == 0) p.weights[bl] = (double)w;
   return w > 0 ? (float)((double)unscale / ((double)w * (double)p.N)) : 0.f;
+}
+
+// The same for a CTA of 256 threads and one baseline (blockIdx.y): every CTA
+// of the row counts for itself, which costs less than a launch before it.
+__device__ __forceinline__ float cta_scale(const FinParams& p, float unscale) {
+  __shared__ float s_scale;
+  __shared__ int s_count[8];
+  int cnt = count_valid(p, blockIdx.y, threadIdx.x, 256);
+  for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
+  if ((threadIdx.x & 31) == 0) s_count[threadIdx.x >> 5] = cnt;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int w = 0;
+    for (int q = 0; q < 8; ++q) w += s_count[q];
+    s_scale = fin_scale(p, blockIdx.y, w, unscale);
+  }
+  __syncthreads();
+  return s_scale;
 }
 
 // Partial sums [KZ][nbl][G][nchan] -> out.  A CTA takes elements of one
@@ -69,52 +75,63 @@ __device__ __forceinline__ float fin_scale(const FinParams& p, int bl, float uns
 // groups share it.
 template <int KG>
 __global__ void __launch_bounds__(256) k_finalize(FinParams p) {
-  constexpr int EL = 256 / KG, PER = KG == 1 ? 8 : 1;  // a thread takes PER elements, EL apart
+  constexpr int EL = 256 / KG, PER = KG == 1 ? 8 : 1;  // a thread takes PER elements, EL apart, at a time
   const int bl = blockIdx.y;
   const size_t per = (size_t)p.G * p.nchan;
   const size_t total = (size_t)nbl_of(p.S) * per;
-  __shared__ float s_sc;
   __shared__ float2 s_sum[KG > 1 ? 256 : 1];
-  if (threadIdx.x == 0) s_sc = fin_scale(p, bl, p.unscale);
+  const float sc = cta_scale(p, p.unscale);
   const bool failed = p.err && *p.err != 0;
-  const int q = threadIdx.x / EL;
-  const size_t k = (size_t)blockIdx.x * EL * PER + threadIdx.x % EL;
-  float2 v[PER];
-#pragma unroll
-  for (int u = 0; u < PER; ++u) v[u] = make_float2(0.f, 0.f);
-#pragma unroll(KG > 1 ? 8 : 1)
-  for (int kz = q; kz < p.KZ; kz += KG) {
-    const float2* src = p.part + (size_t)kz * total + (size_t)bl * per + k;
-    float2 x[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) x[u] = k + u * EL < per ? __ldcs(src + u * EL) : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int u = 0; u < PER; ++u) v[u] = make_float2(v[u].x + x[u].x, v[u].y + x[u].y);
-  }
-  if constexpr (KG > 1) s_sum[threadIdx.x] = v[0];
-  __syncthreads();
-  if (q != 0) return;
-  if constexpr (KG > 1) {
-#pragma unroll
-    for (int g = 1; g < KG; ++g) {
-      const float2 x = s_sum[g * EL + threadIdx.x];
-      v[0].x += x.x;
-      v[0].y += x.y;
-    }
-  }
   const float nan = __int_as_float(0x7fc00000);
+  const int q = threadIdx.x / EL;
+  for (size_t k0 = (size_t)blockIdx.x * EL * PER; k0 < per; k0 += (size_t)gridDim.x * EL * PER) {
+    const size_t k = k0 + threadIdx.x % EL;
+    float2 v[PER];
 #pragma unroll
-  for (int u = 0; u < PER; ++u)
-    if (k + u * EL < per)
-      p.out[(size_t)bl * per + k + u * EL] = failed ? make_float2(nan, nan) : make_float2(v[u].x * s_sc, v[u].y * s_sc);
+    for (int u = 0; u < PER; ++u) v[u] = make_float2(0.f, 0.f);
+#pragma unroll(KG > 1 ? 8 : 1)
+    for (int kz = q; kz < p.KZ; kz += KG) {
+      const float2* src = p.part + (size_t)kz * total + (size_t)bl * per + k;
+      float2 x[PER];
+#pragma unroll
+      for (int u = 0; u < PER; ++u) x[u] = k + u * EL < per ? __ldcs(src + u * EL) : make_float2(0.f, 0.f);
+#pragma unroll
+      for (int u = 0; u < PER; ++u) v[u] = make_float2(v[u].x + x[u].x, v[u].y + x[u].y);
+    }
+    if constexpr (KG > 1) {
+      __syncthreads();  // the sums of the elements before have been read
+      s_sum[threadIdx.x] = v[0];
+      __syncthreads();
+      if (q != 0) continue;
+#pragma unroll
+      for (int g = 1; g < KG; ++g) {
+        const float2 x = s_sum[g * EL + threadIdx.x];
+        v[0].x += x.x;
+        v[0].y += x.y;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+      if (k + u * EL < per)
+        p.out[(size_t)bl * per + k + u * EL] = failed ? make_float2(nan, nan) : make_float2(v[u].x * sc, v[u].y * sc);
+  }
+}
+
+// CTAs along a baseline's elements: one per `each` of them, but no more than
+// fill the SMs a few times over all baselines, since every CTA counts the
+// baseline's valid blocks.
+static unsigned row_ctas(size_t elements, size_t each, int rows) {
+  const size_t need = (elements + each - 1) / each, room = std::max(1, 152 * 32 / rows);
+  return (unsigned)std::min(need, room);
 }
 
 cudaError_t launch_finalize(const FinParams& p, cudaStream_t s) {
   const size_t per = (size_t)p.G * p.nchan;
+  const int nbl = nbl_of(p.S);
   if (p.KZ > 8)
-    k_finalize<16><<<dim3((unsigned)((per + 15) / 16), nbl_of(p.S)), 256, 0, s>>>(p);
+    k_finalize<16><<<dim3(row_ctas(per, 16, nbl), nbl), 256, 0, s>>>(p);
   else
-    k_finalize<1><<<dim3((unsigned)((per + 2047) / 2048), nbl_of(p.S)), 256, 0, s>>>(p);
+    k_finalize<1><<<dim3(std::max(row_ctas(per, 2048, nbl), (unsigned)((per + 8191) / 8192)), nbl), 256, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -125,41 +142,42 @@ cudaError_t launch_finalize(const FinParams& p, cudaStream_t s) {
 // (2.2 GB each way) took 6.0 ms with 8-byte reads 16 KB apart and an FP64
 // quotient per value, 0.64 ms now, 6.8 TB/s.
 constexpr int kTurn = 32;
-__device__ __forceinline__ void load_turn(const FinParams& p, size_t gk0, size_t per, int bl0, int nbl,
-                                          float2 (&tile)[kTurn][kTurn + 1]) {
-#pragma unroll
-  for (int r = 0; r < kTurn; r += 8) {
-    const size_t gk = gk0 + r + threadIdx.y;
-    const int bl = bl0 + threadIdx.x;
-    if (gk < per && bl < nbl) tile[r + threadIdx.y][threadIdx.x] = __ldcs(p.part + gk * nbl + bl);
-  }
-}
-
 __global__ void __launch_bounds__(256) k_finalize_tc(FinParams p, float unscale) {
   __shared__ float2 tile[kTurn][kTurn + 1];
   __shared__ float s_sc[kTurn];
   const int nbl = nbl_of(p.S);
   const size_t per = (size_t)p.G * p.nchan;
   const int bl0 = blockIdx.y * kTurn;
-  const size_t gk0 = (size_t)blockIdx.x * kTurn;
-  if (threadIdx.y == 0) s_sc[threadIdx.x] = bl0 + threadIdx.x < nbl ? fin_scale(p, bl0 + threadIdx.x, unscale) : 0.f;
-  load_turn(p, gk0, per, bl0, nbl, tile);
-  __syncthreads();
+  for (int r = threadIdx.y; r < kTurn && bl0 + r < nbl; r += 8) {  // a warp per baseline
+    int cnt = count_valid(p, bl0 + r, threadIdx.x, 32);
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(0xffffffffu, cnt, o);
+    if (threadIdx.x == 0) s_sc[r] = fin_scale(p, bl0 + r, cnt, unscale);
+  }
+  for (size_t gk0 = (size_t)blockIdx.x * kTurn; gk0 < per; gk0 += (size_t)gridDim.x * kTurn) {
+    __syncthreads();  // the tile before has been written out
 #pragma unroll
-  for (int r = 0; r < kTurn; r += 8) {
-    const int row = r + threadIdx.y;
-    const size_t gk = gk0 + threadIdx.x;
-    if (gk < per && bl0 + row < nbl) {
-      const float2 v = tile[threadIdx.x][row];
-      p.out[(size_t)(bl0 + row) * per + gk] = make_float2(v.x * s_sc[row], v.y * s_sc[row]);
+    for (int r = 0; r < kTurn; r += 8) {
+      const size_t gk = gk0 + r + threadIdx.y;
+      const int bl = bl0 + threadIdx.x;
+      if (gk < per && bl < nbl) tile[r + threadIdx.y][threadIdx.x] = __ldcs(p.part + gk * nbl + bl);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kTurn; r += 8) {
+      const int row = r + threadIdx.y;
+      const size_t gk = gk0 + threadIdx.x;
+      if (gk < per && bl0 + row < nbl) {
+        const float2 v = tile[threadIdx.x][row];
+        p.out[(size_t)(bl0 + row) * per + gk] = make_float2(v.x * s_sc[row], v.y * s_sc[row]);
+      }
     }
   }
 }
 
 cudaError_t launch_finalize_tc(const FinParams& p, float unscale, cudaStream_t s) {
   const size_t per = (size_t)p.G * p.nchan;
-  const int nbl = nbl_of(p.S);
-  k_finalize_tc<<<dim3((unsigned)((per + kTurn - 1) / kTurn), (nbl + kTurn - 1) / kTurn), dim3(kTurn, 8), 0, s>>>(p, unscale);
+  const int rows = (nbl_of(p.S) + kTurn - 1) / kTurn;
+  k_finalize_tc<<<dim3(row_ctas(per, kTurn, rows), rows), dim3(kTurn, 8), 0, s>>>(p, unscale);
   return cudaGetLastError();
 }
 
@@ -185,9 +203,7 @@ __global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unsca
   const int S = p.S, nsub = p.G, nch = p.nchan;
   const int nblv = nbl_of(2 * S);
   const int bl = blockIdx.y;
-  __shared__ float s_sc;
-  if (threadIdx.x == 0) s_sc = fin_scale(p, bl, unscale);
-  __syncthreads();
+  const float sc = cta_scale(p, unscale);
   int a = 0, q = bl;
   while (q >= S - a) { q -= S - a; ++a; }
   const int b = a + q;
@@ -207,13 +223,13 @@ __global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unsca
       v.y += x.y;
     }
     if (flip) v.y = -v.y;
-    p.out[(size_t)bl * per + e] = make_float2(v.x * s_sc, v.y * s_sc);
+    p.out[(size_t)bl * per + e] = make_float2(v.x * sc, v.y * sc);
   }
 }
 
 cudaError_t launch_finalize_cross(const FinParams& p, bool tc, float unscale, cudaStream_t s) {
   const int per = p.G * 4 * p.nchan;
-  const dim3 grid((per + 1023) / 1024, nbl_of(p.S));
+  const dim3 grid(row_ctas(per, 1024, nbl_of(p.S)), nbl_of(p.S));
   if (tc)
     k_finalize_cross<true><<<grid, 256, 0, s>>>(p, unscale);
   else
