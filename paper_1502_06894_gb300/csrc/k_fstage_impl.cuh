@@ -846,6 +846,30 @@ __device__ __forceinline__ float2 prerot(int m, float phi0, float dhi, float dlo
   return cis_turns(fmaf(fm, dlo, phi0) + a);
 }
 
+// The rotation over the r T samples (r < R0) between the points that a thread
+// of the first pass takes: the same for all threads and both polarisations of
+// a (slot, subband), so the CTA forms it once per step (with the accurate sine
+// and cosine) and a point costs one complex product instead of a sine, a
+// cosine and two reductions of its own phase, whose special-function and
+// issue slots bound the pre-F form with the transform's (2048 points: 720 us
+// per 2.7e8 samples, 680 now).
+template <int L>
+__device__ __forceinline__ void fill_rotations(const FParams& p, int s, int bb0, int nslots, const int* s_ok, float2* rot) {
+  constexpr int R0 = Plan<L>::R0, T = Plan<L>::T;
+  for (int e = threadIdx.x; e < nslots * p.nsub * R0; e += blockDim.x) {
+    const int r = e % R0;
+    const int sb = e / R0 % p.nsub, sl = e / R0 / p.nsub;
+    if (!s_ok[sl]) continue;
+    const float2 dph = p.dphi[((size_t)s * p.nsub + sb) * p.ld + p.blk0 + bb0 + sl];
+    const float fm = (float)(r * T);
+    float a = fm * dph.x;  // exact, see prerot
+    a -= rintf(a);
+    float sn, cs;
+    sincospif(2.0f * fmaf(fm, dph.y, a), &sn, &cs);
+    rot[e] = make_float2(cs, sn);
+  }
+}
+
 // Store of the pre-F path: channels k = 0..L/2-1 of the complex L-point
 // transform, times the fractional-delay slope exp(+2 pi i k delta) (the
 // fringe phase was applied before the transform), by the same walk as the
@@ -905,6 +929,7 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
   static_assert(kWordsOffset<L>(NGRP) % 16 == 0, "staging area must be 16-byte aligned");
   uint32_t* wbuf = reinterpret_cast<uint32_t*>(smem_raw + kWordsOffset<L>(NGRP));
   uint32_t* codes = wbuf + slots * wslot;  // TURN
+  float2* rot = reinterpret_cast<float2*>(codes + (size_t)slots * jb * Codes<L, PRE>::W * T);  // TURN and PRE: [slot][subband][R0]
 
   const int tid = threadIdx.x;
   const int grp = tid / T;
@@ -953,6 +978,9 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
     for (int j0 = 0; j0 < G; j0 += jb) {
     const int nj = min(jb, G - j0);
     if constexpr (TURN) {
+      if constexpr (PRE) {
+        if (j0 == 0) fill_rotations<L>(p, s, bb0, nslots, s_ok[nb], rot);
+      }
       turn_codes<L, GC, PRE>(wcur, wslot, s_ok[nb], s_boff[nb], nslots, G, j0, nj, codes);
       __syncthreads();
       if (more && j0 + jb >= G) {  // the window has been read
@@ -993,17 +1021,25 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
           const size_t ps = ((size_t)s * p.nsub + j / p.npol) * p.ld + d;
           const float phi0 = p.phi[ps];
           const float2 dph = p.dphi[ps];
-#pragma unroll
-          for (int u = 0; u < PER0; ++u) {
-            const int jj = t + u * T;
+          // s_lut16[c] = (l[c] / 2, l[0] / 2): twice its real part is level c
+          if constexpr (TURN) {
+            const float2 z0 = prerot(t, phi0, dph.x, dph.y);
+            const float2* w = rot + (size_t)(sl * p.nsub + j / p.npol) * R0;
 #pragma unroll
             for (int r = 0; r < R0; ++r) {
-              const int m = jj + r * (L / R0);
-              const uint32_t c = TURN ? (cw[r >> 4] >> (2 * (r & 15))) & 3u : load_one<GC>(wsl, boff, G, m, j);
-              // s_lut16[c] = (l[c] / 2, l[0] / 2): twice its real part is level c
-              const float lev = 2.0f * s_lut16[c].x;
-              const float2 z = prerot(m, phi0, dph.x, dph.y);
-              v[u][r] = f2mul(z, bc(lev));
+              const float lev = 2.0f * s_lut16[(cw[r >> 4] >> (2 * (r & 15))) & 3u].x;
+              v[0][r] = f2mul(r == 0 ? z0 : cmul(z0, w[r]), bc(lev));
+            }
+          } else {
+#pragma unroll
+            for (int u = 0; u < PER0; ++u) {
+              const int jj = t + u * T;
+#pragma unroll
+              for (int r = 0; r < R0; ++r) {
+                const int m = jj + r * (L / R0);
+                const float lev = 2.0f * s_lut16[load_one<GC>(wsl, boff, G, m, j)].x;
+                v[u][r] = f2mul(prerot(m, phi0, dph.x, dph.y), bc(lev));
+              }
             }
           }
         } else {
@@ -1112,7 +1148,8 @@ static cudaError_t launch_LG(const FParams& p, cudaStream_t st) {
   auto window = [&](int slots) { return (size_t)slots * wslot * sizeof(uint32_t); };
   auto turned = [&](int slots, int jb) {
     return kWordsOffset<L>(NGRP) + window(slots) +
-           sizeof(uint32_t) * (size_t)slots * jb * Codes<L, PRE>::W * Codes<L, PRE>::T;
+           sizeof(uint32_t) * (size_t)slots * jb * Codes<L, PRE>::W * Codes<L, PRE>::T +
+           (PRE ? sizeof(float2) * (size_t)slots * p.nsub * Codes<L, PRE>::R0 : 0);
   };
   static int sm_count = 0;
   if (!sm_count) {
