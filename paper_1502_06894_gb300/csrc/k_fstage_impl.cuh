@@ -179,11 +179,12 @@ __device__ __forceinline__ void twiddle_products(float2 (&v)[R], const float2 (&
 // instead: consecutive k in consecutive words, read after the barrier.
 //
 // stockham_values leaves the results of butterfly group j = t + uT, point
-// (j / NS) NS R + (j mod NS) + r NS, in v[u][r].
-template <int L, int R, int NS, int T, int P, int TWS>
-__device__ __forceinline__ void stockham_values(const float2* __restrict__ buf, int t, int grp,
-                                                const float2* __restrict__ twN, const float2* __restrict__ s_twl,
-                                                const float2* __restrict__ s_twp, float2 (&v)[L / R / T][R]) {
+// (j / NS) NS R + (j mod NS) + r NS, in v[u][r].  `load(u, r)` reads its point
+// j + r L/R, `loaded()` follows the reads.
+template <int L, int R, int NS, int T, int TWS, typename Load, typename Loaded>
+__device__ __forceinline__ void stockham_values(Load load, Loaded loaded, int t, const float2* __restrict__ twN,
+                                                const float2* __restrict__ s_twl, const float2* __restrict__ s_twp,
+                                                float2 (&v)[L / R / T][R]) {
   constexpr int GROUPS = L / R;
   constexpr int PER = GROUPS / T;
   constexpr int LOGR = ilog2c(R);
@@ -200,12 +201,10 @@ __device__ __forceinline__ void stockham_values(const float2* __restrict__ buf, 
     }
   }
 #pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const int j = t + u * T;
+  for (int u = 0; u < PER; ++u)
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[u][r] = buf[padp<P>(j + r * GROUPS)];
-  }
-  gsync<T>(grp);
+    for (int r = 0; r < R; ++r) v[u][r] = load(u, r);
+  loaded();
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int k = (t + u * T) & (NS - 1);
@@ -230,7 +229,8 @@ __device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, i
                                               const float2* __restrict__ s_twp = nullptr) {
   constexpr int PER = L / R / T;
   float2 v[PER][R];
-  stockham_values<L, R, NS, T, P, TWS>(buf, t, grp, twN, s_twl, s_twp, v);
+  stockham_values<L, R, NS, T, TWS>([&](int u, int r) { return buf[padp<P>(t + u * T + r * (L / R))]; },
+                                    [&] { gsync<T>(grp); }, t, twN, s_twl, s_twp, v);
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int j = t + u * T;
@@ -239,6 +239,17 @@ __device__ __forceinline__ void stockham_pass(float2* __restrict__ buf, int t, i
     for (int r = 0; r < R; ++r) buf[padp<P>(idxD + r * NS)] = v[u][r];
   }
   gsync<T>(grp);
+}
+
+// Where a three-pass transform keeps the points between its second and third
+// pass.  The second pass writes each result back to the place that it read the
+// operand of the same number from, which no other thread touches: no barrier
+// between its reads and its writes.  Butterfly group j2 = t + uT of the third
+// pass finds its operand r at
+template <int L, int R0, int R1, int T>
+__device__ __forceinline__ int third_place(int t, int u, int r) {
+  static_assert(T % R0 == 0, "places");
+  return padp<R0>(r * R0 + (t & (R0 - 1)) + (t / R0 + (T / R0) * u) * (L / R1));
 }
 
 // FFT plans: L = N/2 complex points; radices R0*R1*R2 = L; T threads per FFT.
@@ -488,6 +499,49 @@ __device__ __forceinline__ void split_rotate_shuffle(const float2 (&z_)[PER][R],
     if (q > 0 || t != 0) store_spec<OUT>(out, obase + (L - k), cmul(Xb, y), scale);
     z = walk(z, cm1, sn);
     y = walk(y, cm1, -sn);
+  }
+  if (t == 0) {  // k = L/2: X = E + W_N^{N/4} O; z has walked to it
+    float2 Xa, Xb;
+    split_values(v(Q / 2), v(Q / 2), make_float2(0.f, -1.f), Xa, Xb);
+    store_spec<OUT>(out, obase + L / 2, cmul(Xa, z), scale);
+  }
+}
+
+// The same for a transform of several warps and three passes: the thread's own
+// results v[u][r] = Z[t + (r PER + u) T] stay in registers, the upper half of
+// them also goes to the places that its operands came from, where the thread
+// of the partner channels reads them.  (Writing and reading all results, with
+// barriers around every pass's writes, took six barriers a transform where
+// this takes four: 2.7e8 samples of 4096-point transforms 510 us, 475 now, of
+// 2048-point ones 434 and 418, pre-F 680 and 647.)
+template <int L, int R0, int R1, int T, int OUT, int PER, int R>
+__device__ __forceinline__ void split_rotate_places(const float2 (&z_)[PER][R], float2* __restrict__ fbuf, int t, int grp,
+                                                    const float2* __restrict__ twN, float phi, float delta, void* out,
+                                                    size_t obase, float scale) {
+  constexpr int Q = L / T;
+  static_assert(PER * R == Q, "last pass");
+  auto v = [&](int q) { return z_[q % PER][q / PER]; };  // Z[t + q T]
+#pragma unroll
+  for (int q = Q / 2; q < Q; ++q) fbuf[third_place<L, R0, R1, T>(t, q % PER, q / PER)] = v(q);
+  gsync<T>(grp);
+  const int tp = (T - t) & (T - 1);  // thread of Z[L - k], element Q - 1 - q (Q - q for thread 0)
+  float2 z = cis_turns(fmaf((float)t, delta, phi));
+  float2 y = cis_turns(fmaf((float)(L - t), delta, phi));
+  float cm1, sn;
+  walk_step((float)T * delta, cm1, sn);
+  SplitTw<L, T> tw(nullptr, twN, t);
+#pragma unroll
+  for (int q = 0; q < Q / 2; ++q) {
+    const int k = t + q * T;
+    const int qp = Q - 1 - q + (t == 0 ? 1 : 0);
+    const float2 Zm = q == 0 && t == 0 ? v(0) : fbuf[third_place<L, R0, R1, T>(tp, qp % PER, qp / PER)];
+    float2 Xa, Xb;
+    split_values(v(q), Zm, tw.get(nullptr, k), Xa, Xb);
+    store_spec<OUT>(out, obase + k, cmul(Xa, z), scale);
+    if (q > 0 || t != 0) store_spec<OUT>(out, obase + (L - k), cmul(Xb, y), scale);
+    z = walk(z, cm1, sn);
+    y = walk(y, cm1, -sn);
+    tw.next();
   }
   if (t == 0) {  // k = L/2: X = E + W_N^{N/4} O; z has walked to it
     float2 Xa, Xb;
@@ -920,8 +974,9 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
   constexpr int R0 = P::R0;
   constexpr int PER0 = L / R0 / T;
   // the last pass's results stay in registers: the pre-F form's store needs only a thread's own,
-  // the real split those of another thread, which a shuffle reaches within a warp
-  constexpr bool REGS = PRE || (T <= 32 && Tw<L>::on && P::R1 > 1 && P::R2 == 1);
+  // the real split half of another thread's, by a shuffle within a warp or through shared memory
+  // (8192 points, 32 a thread at 8 warps per SM: 590 us so, 575 with all results in shared memory)
+  constexpr bool REGS = PRE || (T <= 32 && Tw<L>::on && P::R1 > 1) || (P::R2 > 1 && L <= 4096);
   static_assert(PER0 >= 1, "plan");
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1074,12 +1129,26 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
         const float2* twp1 = PassTw<L>::on ? s_twp : nullptr;
         const float2* twp2 = PassTw<L>::on ? s_twp + PassTw<L>::n1 : nullptr;
         if constexpr (P::R1 > 1) gsync<T>(grp);
-        if constexpr (P::R2 > 1) stockham_pass<L, P::R1, P::R0, T, P::R0, TWS>(fbuf, t, grp, p.twN, nullptr, twp1);
+        if constexpr (P::R2 > 1 && REGS) {  // the second of three passes, in place
+          constexpr int R = P::R1, PER = L / R / T;
+          float2 w[PER][R];
+          stockham_values<L, R, P::R0, T, TWS>([&](int u, int r) { return fbuf[padp<R0>(t + u * T + r * (L / R))]; }, [] {}, t,
+                                               p.twN, nullptr, twp1, w);
+#pragma unroll
+          for (int u = 0; u < PER; ++u)
+#pragma unroll
+            for (int r = 0; r < R; ++r) fbuf[padp<R0>(t + u * T + r * (L / R))] = w[u][r];
+          gsync<T>(grp);
+        }
         if constexpr (REGS) {
-          float2 z[PERL][RL];
-          if constexpr (P::R1 > 1) {
-            stockham_values<L, RL, L / RL, T, P::R0, TWS>(fbuf, t, grp, p.twN, twl, P::R2 > 1 ? twp2 : twp1, z);
-            // Z[t + q T] = z[q % PERL][q / PERL]
+          float2 z[PERL][RL];  // Z[t + q T] = z[q % PERL][q / PERL]
+          if constexpr (P::R2 > 1) {
+            stockham_values<L, RL, L / RL, T, TWS>(
+                [&](int u, int r) { return fbuf[third_place<L, R0, P::R1, T>(t, u, r)]; }, [] {}, t, p.twN, twl, twp2, z);
+          } else if constexpr (P::R1 > 1) {
+            stockham_values<L, RL, L / RL, T, TWS>(
+                [&](int u, int r) { return fbuf[padp<R0>(t + u * T + r * (L / RL))]; }, [&] { gsync<T>(grp); }, t, p.twN, twl,
+                twp1, z);
           } else {
 #pragma unroll
             for (int r = 0; r < RL; ++r) z[0][r] = v[0][r];
@@ -1088,6 +1157,8 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
             constexpr int OUT = decltype(kind)::value;
             if constexpr (PRE)
               rotate_store_pre<L, T, OUT>([&](int q) { return z[q % PERL][q / PERL]; }, t, delta, p.out, obase, p.scale);
+            else if constexpr (P::R2 > 1)
+              split_rotate_places<L, R0, P::R1, T, OUT>(z, fbuf, t, grp, p.twN, phi, delta, p.out, obase, p.scale);
             else
               split_rotate_shuffle<L, T, OUT>(z, s_tw, t, phi, delta, p.out, obase, p.scale);
           };
@@ -1095,6 +1166,7 @@ k_fstage(FParams p, int slots, int wslot, int nseq, int jb) {
           else if (p.out_kind == 2) finish(std::integral_constant<int, 2>{});
           else finish(std::integral_constant<int, 0>{});
         } else if constexpr (P::R1 > 1) {
+          if constexpr (P::R2 > 1) stockham_pass<L, P::R1, P::R0, T, P::R0, TWS>(fbuf, t, grp, p.twN, nullptr, twp1);
           stockham_pass<L, RL, L / RL, T, P::R0, TWS>(fbuf, t, grp, p.twN, twl, P::R2 > 1 ? twp2 : twp1);
         } else {
           gsync<T>(grp);
