@@ -755,7 +755,7 @@ def main():
         roof = {"bound": "alu", "achieved": tfl, "peak": peak_alu / 1e12, "unit": "TFLOP/s", "frac": alu_frac,
                 "traffic": None, "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2 x 2070 MHz"}
     gc = G if G in (16, 32) else 0
-    kname = "k_fstage<%d,%d>" % (nch, gc) if dom == "fstage" else "k_xmac_tma<%d>" % S
+    kname = "k_fstage<%d,%d>" % (nch, gc) if dom == "fstage" else "k_xmac<%d>" % S
     traffic = traffic_per_launch(kname)
     roof["traffic"] = traffic
     roof["traffic_over_algorithmic"] = (traffic / (d_bytes / max(d_n, 1))) if traffic else None
@@ -767,7 +767,7 @@ def main():
     inst = profile_value("instructions.txt", kname)
     roof["warp_instructions"] = inst
     roof["issue_frac"] = issue_frac(inst, t_launch, (clocks or {}).get("sm_mhz") or MAX_SM_MHZ)
-    launches = prof_ovl["delay"][1] + prof_ovl["fstage"][1] + prof_ovl["xstage"][1] + 2 * prof_ovl["finalize"][1]
+    launches = prof_ovl["delay"][1] + prof_ovl["fstage"][1] + prof_ovl["xstage"][1] + prof_ovl["finalize"][1]
     x_tflops = x_flops / (x_ms / 1e3) / 1e12 if x_ms > 0 else None
     def tc_leg(ms_t, prof_t, clocks_t, dtype, elem_bytes, bound, unit, sq):
         xt_ms, xt_n = prof_t["xstage"]

@@ -359,11 +359,12 @@ int corr_launch_shape(const corr_t *h, int *chunk_blocks, int *kz);
  * the largest |M|, the smaller flat index r * pad_delay + l on ties; its rate
  * bin, lag, amplitude and complex value (2 floats) go to the host pointers
  * (each may be NULL).  pad_rate >= nsub and pad_delay >= nchan are powers of
- * two <= 16384 with pad_rate * pad_delay <= 2^26 (else CORR_EINVAL).  Work
- * space (pad_delay * nsub complex values) is taken with cudaMallocAsync on
- * cuda_stream (NULL: the legacy default stream) and released there
- * (CORR_ENOMEM if that fails); the call returns when the search is done
- * (CORR_ECUDA on a CUDA error). */
+ * two <= 16384 with pad_rate * pad_delay <= 2^26 (else CORR_EINVAL).  The work
+ * runs on cuda_stream (NULL: the legacy default stream) with the map as its
+ * work space; visibilities that lie inside the map themselves need pad_delay *
+ * nsub complex values taken there with cudaMallocAsync and released (CORR_ENOMEM
+ * if that fails).  The call returns when the search is done (CORR_ECUDA on a
+ * CUDA error). */
 int corr_fringe_search(const float *dev_vis, int nsub, int nchan, int pad_rate, int pad_delay, float *dev_map,
                        int *peak_rate, int *peak_lag, float *peak_amp, float *peak_value, void *cuda_stream);
 
@@ -398,8 +399,8 @@ int corr_fringe_search(const float *dev_vis, int nsub, int nchan, int pad_rate, 
  * with small kernels (their values travel as kernel parameters), and only
  * enqueues the work on cuda_stream (NULL: the legacy default stream) before
  * it returns.  All calls share the one array, which keeps the last call's
- * contents (the partial sums and a timeout flag are cleared at the start of
- * every call): calls whose device work overlaps -- on two streams, or from
+ * contents (every call writes its partial sums anew and clears a timeout flag
+ * at its start): calls whose device work overlaps -- on two streams, or from
  * two threads -- race and give wrong results.  Errors are reported by return
  * code only; a device wait of the X step that runs out of time (see
  * CORR_ETIMEOUT) cannot be reported that way, since the call has returned by
