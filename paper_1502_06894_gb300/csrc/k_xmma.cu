@@ -383,10 +383,15 @@ cudaError_t launch_xtc2(const XTC2Params& p_in, int sm_count, cudaStream_t s) {
 // share an SM, so that one writes while the others read.  All stations of 64
 // in one CTA left room for 8 E4M3 or 4 FP16 channels, 16 bytes of each 32-byte
 // sector (64 stations x 32 streams x 4096 channels x 512 blocks of
-// E4M3: 5.46 ms, 3.98 now; 17 x 7 x 2048 x 512 of FP16: 273 and 178 us).
+// E4M3: 5.46 ms, 3.81 now; 17 x 7 x 2048 x 512 of FP16: 273 and 174 us).
 constexpr int kTurnRow = 144;   // bytes per staged row (128 bytes of values + 16 bytes of padding)
 constexpr int kTurnRows = 512;  // staged rows per CTA: 2 (Re, Im) x stations x channels
 template <bool FP8> constexpr int kTurnCh = FP8 ? 32 : 16;  // channels per CTA: 64 bytes of a spectrum
+
+// A staged row starts this many of its eight 16-byte chunks later (cyclically):
+// the threads that store one block's channels, 8 (E4M3) or 4 (FP16) rows apart,
+// would otherwise meet in the same banks (rows are multiples of 16 bytes apart).
+__device__ __forceinline__ int turn_rot(int c) { return 2 * (c >> 3); }
 
 // Write phase: stations [s0, s0 + ns).
 template <int CH>
@@ -408,7 +413,7 @@ __device__ __forceinline__ void write_staged_rows(const unsigned char* turn_raw,
   for (int rs = threadIdx.x / per; rs < 2 * ns; rs += blockDim.x / per) {
     const int ri = rs >= ns ? 1 : 0;
     const int s = rs - ri * ns;
-    const uint4 v = *reinterpret_cast<const uint4*>(turn_raw + ((size_t)rs * CH + c) * kTurnRow + kc * 16);
+    const uint4 v = *reinterpret_cast<const uint4*>(turn_raw + ((size_t)rs * CH + c) * kTurnRow + ((kc + turn_rot(c)) & 7) * 16);
     const int r = (cl * S + s0 + s) * 2 + ri;
     *reinterpret_cast<uint4*>(tile + (r >> 3) * 1024 + (r & 7) * 128 + ((kc ^ (r & 7)) << 4)) = v;
   }
@@ -485,14 +490,14 @@ __global__ void __launch_bounds__(256) k_tiles(const unsigned char* __restrict__
         if constexpr (FP8) {
           // channel e sits in bytes 0,1 (even e) or 2,3 (odd e) of its word
           const uint32_t sre = (e & 1) ? 0x0062u : 0x0040u, sim = (e & 1) ? 0x0073u : 0x0051u;
-          *reinterpret_cast<uint32_t*>(re_row + e * kTurnRow + 4 * b4) =
+          *reinterpret_cast<uint32_t*>(re_row + e * kTurnRow + 4 * ((b4 + 4 * turn_rot(c)) & 31)) =
               __byte_perm(__byte_perm(w[0], w[1], sre), __byte_perm(w[2], w[3], sre), 0x5410);
-          *reinterpret_cast<uint32_t*>(im_row + e * kTurnRow + 4 * b4) =
+          *reinterpret_cast<uint32_t*>(im_row + e * kTurnRow + 4 * ((b4 + 4 * turn_rot(c)) & 31)) =
               __byte_perm(__byte_perm(w[0], w[1], sim), __byte_perm(w[2], w[3], sim), 0x5410);
         } else {
-          *reinterpret_cast<uint2*>(re_row + e * kTurnRow + 8 * b4) =
+          *reinterpret_cast<uint2*>(re_row + e * kTurnRow + 8 * ((b4 + 2 * turn_rot(c)) & 15)) =
               make_uint2(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410));
-          *reinterpret_cast<uint2*>(im_row + e * kTurnRow + 8 * b4) =
+          *reinterpret_cast<uint2*>(im_row + e * kTurnRow + 8 * ((b4 + 2 * turn_rot(c)) & 15)) =
               make_uint2(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632));
         }
       }
