@@ -338,8 +338,10 @@ int corr_set_profiling(corr_t *h, int enable);
  * (ms) and the number of launches since the last read, and reset them. */
 int corr_read_profile(corr_t *h, double ms[4], int64_t launches[4]);
 
-/* Blocks per F/X chunk and the number of X partial accumulators the handle
- * uses (valid after the first correlate call). */
+/* Blocks per F/X chunk (the most; unless corr_set_chunk_blocks chose them, an
+ * integration is cut into equal chunks of at most that many) and the number of
+ * X partial accumulators the handle uses (valid after the first correlate
+ * call). */
 int corr_launch_shape(const corr_t *h, int *chunk_blocks, int *kz);
 
 /* ---- delay-rate fringe search ---------------------------------------------
