@@ -3,8 +3,10 @@
 //
 // One CTA takes one station and a few FFT blocks.  Per block it stages the
 // packed 2-bit words of the delay-tracked window [b*N + n_b, +N) in shared
-// memory once (all G streams of a station share one window), then each
-// FFT group of T threads transforms one stream:
+// memory once (all G streams of a station share one window), turns their codes
+// into words per stream (transforms of 64 to 4096 points), then each FFT group
+// of T threads transforms one stream (k_fstage_impl.cuh; this file holds the
+// dispatch and the tensor-core variant):
 //
 //   unpack   2-bit codes -> levels, two real samples per complex point through
 //            one 16-entry table of level pairs (pre-halved, which absorbs the
