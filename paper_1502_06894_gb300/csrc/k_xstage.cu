@@ -15,6 +15,7 @@
 // add per element and launch, so results are deterministic and the FP32 sums
 // stay short (hierarchical accumulation).
 #include "corr_internal.cuh"
+#include "ring_log.h"
 
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -109,7 +110,8 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, volati
 // 1.58 ms; warp 0 refilling each time 1.69, slot q - 1 instead 2.33).
 struct Ring {
   uint64_t *full, *empty;
-  volatile int *abort_flag, *issued;  // `issued`: stages whose copies were issued, in order
+  volatile int* abort_flag;
+  RingLog<kMaxStages>* log;  // the copies issued
   int stages;
   long long limit;
 
@@ -121,14 +123,15 @@ struct Ring {
       }
       asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
       *abort_flag = 0;
-      *issued = 0;
+      log->clear();
     }
     __syncthreads();
   }
-  // at stage q, held in `slot` with parity `phase`: the place of stage q - 2, once every warp has read it (-1: gave up)
+  // at stage q, held in `slot` with parity `phase`: the place of stage q - 2, once every warp has read it (-1: gave
+  // up, here or in another warp before)
   __device__ __forceinline__ int reclaim(int slot, uint32_t phase) const {
     const int old = slot >= 2 ? slot - 2 : slot - 2 + stages;
-    if (ring_wait(&empty[old], old > slot ? phase ^ 1 : phase, abort_flag, limit)) return old;
+    if (!*abort_flag && ring_wait(&empty[old], old > slot ? phase ^ 1 : phase, abort_flag, limit) && !*abort_flag) return old;
     *abort_flag = 1;
     return -1;
   }
@@ -141,10 +144,10 @@ struct Ring {
   // After an abort, with every warp of the CTA past its last issue: let the
   // copies in flight land before the CTA's shared memory goes away.
   __device__ __forceinline__ void drain(int* err) const {
-    const int n = *issued;
-    for (int q = n > stages ? n - stages : 0; q < n; ++q)
+    log->for_each(stages, [&](int slot, unsigned parity) {
       for (long long it = 0; it < kXDrainLimit; ++it)
-        if (ring_poll(&full[q % stages], (uint32_t)((q / stages) & 1))) break;
+        if (ring_poll(&full[slot], parity)) break;
+    });
     if (err) atomicExch(err, 1);
   }
 };
@@ -220,7 +223,8 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
   extern __shared__ __align__(128) unsigned char ring_raw[];
   unsigned char* data = ring_raw + ((128u - (xs_u32(ring_raw) & 127u)) & 127u);
   __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
-  __shared__ volatile int s_abort, s_issued;
+  __shared__ volatile int s_abort;
+  __shared__ RingLog<kMaxStages> s_log;
   constexpr int EB = spec_bytes(IN);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int k0 = blockIdx.x * 32 * sh.cg;
@@ -231,7 +235,7 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
   if (b_hi <= b_lo && !p.first) return;  // an empty range of the first chunk writes zeros
   const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
   const int row_bytes = sh.pitch * EB;
-  Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
+  Ring ring{s_full, s_empty, &s_abort, &s_log, sh.nst, p.wait_limit};
   ring.init(sh.cg);
   auto issue = [&](int q, int slot) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xs_u32(&s_full[slot])),
@@ -243,7 +247,7 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
         "l"(reinterpret_cast<uint64_t>(&tmap)), "r"(2 * k0), "r"(0), "r"(g * p.CB + b_lo + q * sh.nb),
         "r"(xs_u32(&s_full[slot]))
         : "memory");
-    s_issued = q + 1;
+    s_log.note(slot, q);
   };
   if (threadIdx.x == 0)
     for (int q = 0; q < sh.nst && q < nst; ++q) issue(q, q);
@@ -309,7 +313,8 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
   extern __shared__ __align__(128) unsigned char ring_raw[];
   unsigned char* data = ring_raw + ((128u - (xs_u32(ring_raw) & 127u)) & 127u);
   __shared__ __align__(8) uint64_t s_full[kMaxStages], s_empty[kMaxStages];
-  __shared__ volatile int s_abort, s_issued;
+  __shared__ volatile int s_abort;
+  __shared__ RingLog<kMaxStages> s_log;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const XGroup& gr = groups.g[blockIdx.x % groups.n];
   const int k0 = blockIdx.x / groups.n * 32;
@@ -319,7 +324,7 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
   if (b_hi <= b_lo && !p.first) return;  // an empty range of the first chunk writes zeros
   const int nst = (b_hi - b_lo + sh.nb - 1) / sh.nb;
   const int row_bytes = sh.pitch * 8, nwarp = gr.nwarp;
-  Ring ring{s_full, s_empty, &s_abort, &s_issued, sh.nst, p.wait_limit};
+  Ring ring{s_full, s_empty, &s_abort, &s_log, sh.nst, p.wait_limit};
   ring.init(nwarp);
   auto issue = [&](int q, int slot) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(xs_u32(&s_full[slot])),
@@ -332,7 +337,7 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
           "l"(reinterpret_cast<uint64_t>(&tmap)), "r"(2 * k0), "r"((int)gr.tile[i] * TS),
           "r"(g * p.CB + b_lo + q * sh.nb), "r"(xs_u32(&s_full[slot]))
           : "memory");
-    s_issued = q + 1;
+    s_log.note(slot, q);
   };
   if (threadIdx.x == 0)
     for (int q = 0; q < sh.nst && q < nst; ++q) issue(q, q);
