@@ -17,7 +17,37 @@
 
 namespace corr {
 
-cudaError_t fringe_init_constants() { return init_w32(); }
+namespace {
+
+// What FP32 leaves of c_w32 and c_w32n: exp(-2 pi i m / 32) to twice the bits.
+__constant__ float2 c_w32_low[32];
+__constant__ float2 c_w32n_low[32];
+
+// a W_32^m with the constant's low part: rounded like a product by the exact
+// root.  The few constants of a 32-point butterfly meet every value of a
+// transform, so their own roundings would not average out: with FP32 constants
+// alone a search is less exact than one of radix-2 passes.
+struct TurnW32Exact {
+  __device__ __forceinline__ float2 operator()(float2 a, int m) const {
+    const float2 low = f2fma(swp(a), c_w32n_low[m], f2mul(a, bc(c_w32_low[m].x)));
+    return f2fma(swp(a), c_w32n[m], f2fma(a, bc(c_w32[m].x), low));
+  }
+};
+
+}  // namespace
+
+cudaError_t fringe_init_constants() {
+  cudaError_t e = init_w32();
+  if (e != cudaSuccess) return e;
+  float2 h[32], hn[32];
+  for (int m = 0; m < 32; ++m) {
+    const double a = -2.0 * 3.14159265358979323846 * (double)m / 32.0;
+    h[m] = make_float2((float)(cos(a) - (double)(float)cos(a)), (float)(sin(a) - (double)(float)sin(a)));
+    hn[m] = make_float2(-h[m].y, h[m].y);
+  }
+  if ((e = cudaMemcpyToSymbol(c_w32_low, h, sizeof(h))) != cudaSuccess) return e;
+  return cudaMemcpyToSymbol(c_w32n_low, hn, sizeof(hn));
+}
 
 namespace {
 
@@ -64,21 +94,31 @@ __device__ __forceinline__ int at(int i, int c) {
   else return c * (n + n / Radices<n>::R0 + 1) + padp<Radices<n>::R0>(i);
 }
 
-// v[r] *= W_{NS R}^{-k r}: the powers k 2^i from sincospif, whose argument is
-// exact, and the rest as their products.  The transforms work on swapped
-// (imaginary, real) values, which turns the forward butterflies of dft_reg
-// into inverse ones, so the twiddles here are the forward ones.
+// v[r] *= W_{NS R}^{-k r}.  r splits into its low bits a and its high bits b:
+// W^{k a} and W^{k b} come from sincospif, whose argument is exact, and a
+// factor is one product of the two at most (ten sines and cosines for 32
+// points; with the powers k 2^i alone, five, a factor is up to four roundings
+// away and the search less exact than one of radix-2 passes).  The transforms
+// work on swapped (imaginary, real) values, which turns the forward butterflies
+// of dft_reg into inverse ones, so the twiddles here are the forward ones.
 template <int R, int NS>
 __device__ __forceinline__ void cfft_twiddle(float2 (&v)[R], int k) {
-  constexpr int LOGR = ilog2c(R);
-  float2 wp[LOGR];
-#pragma unroll
-  for (int i = 0; i < LOGR; ++i) {
+  constexpr int LO = ilog2c(R) / 2, NA = 1 << LO, NB = R / NA;
+  auto root = [&](int r) {
     float sn, cs;
-    sincospif(-2.0f * (float)(k << i) / (float)(NS * R), &sn, &cs);
-    wp[i] = make_float2(cs, sn);
+    sincospif(-2.0f * (float)(k * r) / (float)(NS * R), &sn, &cs);
+    return make_float2(cs, sn);
+  };
+  float2 A[NA];
+#pragma unroll
+  for (int a = 1; a < NA; ++a) A[a] = root(a);
+#pragma unroll
+  for (int b = 0; b < NB; ++b) {
+    const float2 B = b ? root(b * NA) : make_float2(1.f, 0.f);
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+      if (a || b) v[b * NA + a] = cmul(v[b * NA + a], a && b ? cmul(A[a], B) : a ? A[a] : B);
   }
-  twiddle_products<R, LOGR>(v, wp);
 }
 
 // A middle or last pass: R points a butterfly from shared memory; the middle
@@ -97,7 +137,7 @@ __device__ __forceinline__ void cfft_pass(float2* buf, int t, int c, Store store
   for (int u = 0; u < PER; ++u) {
     const int j = t + u * T, k = j & (NS - 1);
     cfft_twiddle<R, NS>(v[u], k);
-    dft_reg<R>(v[u]);
+    dft_reg<R>(v[u], TurnW32Exact());
 #pragma unroll
     for (int r = 0; r < R; ++r) {
       if constexpr (last) store(k + r * NS, v[u][r]);
@@ -163,7 +203,7 @@ k_cfft_inv(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out
     }
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
-    dft_reg<P::R0>(v[u]);
+    dft_reg<P::R0>(v[u], TurnW32Exact());
 #pragma unroll
     for (int r = 0; r < P::R0; ++r) {
       if constexpr (P::R1 == 1) store(r, v[u][r]);

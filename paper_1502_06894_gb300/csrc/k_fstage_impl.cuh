@@ -59,9 +59,11 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return f2fma(swp(a), make_float2(-b.y, b.y), f2mul(a, bc(b.x)));
 }
 // a W_32^m, the second operand pair read ready-made from c_w32n
-__device__ __forceinline__ float2 cmul_w32(float2 a, int m) {
-  return f2fma(swp(a), c_w32n[m], f2mul(a, bc(c_w32[m].x)));
-}
+struct TurnW32 {
+  __device__ __forceinline__ float2 operator()(float2 a, int m) const {
+    return f2fma(swp(a), c_w32n[m], f2mul(a, bc(c_w32[m].x)));
+  }
+};
 
 // Shared FFT buffers insert one padding element after every P elements (P =
 // the first pass's radix): pass 0 stores each thread's P outputs contiguously,
@@ -75,9 +77,9 @@ __device__ __forceinline__ int padp(int i) { return i + (i >> ilog2c(P)); }
 // multiply-add that its butterfly needs anyway (the product by +-1 is exact, so
 // the rounding is that of the rotation and the addition), which takes 228
 // packed instructions for 32 points instead of 243, the bound of this routine
-// (two cycles each: 491 -> 460 cycles).
-template <int R>
-__device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
+// (two cycles each: 491 -> 460 cycles).  `turn(d, m)` is d W_32^m.
+template <int R, typename Turn = TurnW32>
+__device__ __forceinline__ void dft_reg(float2 (&v)[R], Turn turn = Turn()) {
   constexpr int LOG = ilog2c(R);
 #pragma unroll
   for (int st = 0; st < LOG; ++st) {
@@ -93,7 +95,7 @@ __device__ __forceinline__ void dft_reg(float2 (&v)[R]) {
         v[i + k] = turned ? f2fma(swp(b), pm, a) : f2add(a, b);
         const float2 d = turned ? f2fma(swp(b), mp, a) : f2sub(a, b);
         const int m = k * (32 / (2 * half));  // W_{2 half}^k = W_32^m
-        v[i + k + half] = (m == 0 || m == 8) ? d : cmul_w32(d, m);
+        v[i + k + half] = (m == 0 || m == 8) ? d : turn(d, m);
       }
     }
   }
