@@ -1291,10 +1291,13 @@ int corr_reset(corr_t* h) {
   if (!h) return CORR_EINVAL;
   int rc = use_device(h);
   if (rc) return rc;
-  cudaStreamSynchronize(h->stream);
-  if (h->xstream) cudaStreamSynchronize(h->xstream);
-  drop_lookahead(h);
-  drain_pushes(h);
+  // the handle is reset whatever these waits return; an error is reported at the end
+  cudaError_t e = cudaStreamSynchronize(h->stream);
+  if (h->xstream) {
+    const cudaError_t ex = cudaStreamSynchronize(h->xstream);
+    if (e == cudaSuccess) e = ex;
+  }
+  const int rc_ahead = drop_lookahead(h), rc_push = drain_pushes(h);
   for (Station& s : h->st) {
     for (auto& pe : s.pending) cudaEventDestroy(pe.ev);
     s.pending.clear();
@@ -1311,9 +1314,12 @@ int corr_reset(corr_t* h) {
   }
   h->flushed = false;
   h->next_int = 0;
-  // a device wait that timed out earlier no longer blocks the handle
   if (h->prepared) {
-    *h->h_err = 0;
+    if (e != cudaSuccess || rc_ahead || rc_push) {
+      cudaGetLastError();  // not for the next launch to report
+      return e != cudaSuccess ? h->cuda_fail(e, "corr_reset: waiting for the handle's work") : rc_ahead ? rc_ahead : rc_push;
+    }
+    *h->h_err = 0;  // a device wait that timed out earlier no longer blocks the handle
   }
   return CORR_OK;
 }
