@@ -83,6 +83,9 @@ template <int n> struct Radices {
 template <int n, bool COLS> struct Batch {
   static constexpr int T = Radices<n>::T;
   static constexpr int C = T >= 256 ? 1 : COLS ? (n <= 64 ? 128 / T : n <= 256 ? 32 : 8192 / n) : 256 / T > 64 ? 64 : 256 / T;
+  // complex values in shared memory: the points (rows padded, see at()), and the second pass's twiddles
+  static constexpr int POINTS = Radices<n>::R1 == 1 ? 0 : COLS ? n * C : C * (n + n / Radices<n>::R0 + 1);
+  static constexpr int TWIDDLES = Radices<n>::R0 * (Radices<n>::R1 - 1);
 };
 
 // Position of point i of transform c in shared memory: columns side by side
@@ -94,27 +97,36 @@ __device__ __forceinline__ int at(int i, int c) {
   else return c * (n + n / Radices<n>::R0 + 1) + padp<Radices<n>::R0>(i);
 }
 
-// v[r] *= W_{NS R}^{-k r}.  r splits into its low bits a and its high bits b:
-// W^{k a} and W^{k b} come from sincospif, whose argument is exact, and a
-// factor is one product of the two at most (ten sines and cosines for 32
-// points; with the powers k 2^i alone, five, a factor is up to four roundings
-// away and the search less exact than one of radix-2 passes).  The transforms
+// W_N^m, rounded once: sincospif of an argument that is exact.  The transforms
 // work on swapped (imaginary, real) values, which turns the forward butterflies
 // of dft_reg into inverse ones, so the twiddles here are the forward ones.
-template <int R, int NS>
-__device__ __forceinline__ void cfft_twiddle(float2 (&v)[R], int k) {
+template <int N>
+__device__ __forceinline__ float2 root(int m) {
+  float sn, cs;
+  sincospif(-2.0f * (float)m / (float)N, &sn, &cs);
+  return make_float2(cs, sn);
+}
+
+// v[r] *= W_{NS R}^{k r}.  The second pass has few k, so the CTA forms all its
+// factors once, [r - 1][k] in `table`.  The third pass has one k a butterfly: r
+// splits into its low bits a and its high bits b, and a factor is one product of
+// W^{k a} and W^{k b} at most (ten sines and cosines for 32 points; with the
+// powers k 2^i alone, five, a factor is up to four roundings away and the search
+// less exact than one of radix-2 passes).
+template <int R, int NS, bool TABLE>
+__device__ __forceinline__ void cfft_twiddle(float2 (&v)[R], int k, const float2* table) {
+  if constexpr (TABLE) {
+#pragma unroll
+    for (int r = 1; r < R; ++r) v[r] = cmul(v[r], table[(r - 1) * NS + k]);
+    return;
+  }
   constexpr int LO = ilog2c(R) / 2, NA = 1 << LO, NB = R / NA;
-  auto root = [&](int r) {
-    float sn, cs;
-    sincospif(-2.0f * (float)(k * r) / (float)(NS * R), &sn, &cs);
-    return make_float2(cs, sn);
-  };
   float2 A[NA];
 #pragma unroll
-  for (int a = 1; a < NA; ++a) A[a] = root(a);
+  for (int a = 1; a < NA; ++a) A[a] = root<NS * R>(k * a);
 #pragma unroll
   for (int b = 0; b < NB; ++b) {
-    const float2 B = b ? root(b * NA) : make_float2(1.f, 0.f);
+    const float2 B = b ? root<NS * R>(k * b * NA) : make_float2(1.f, 0.f);
 #pragma unroll
     for (int a = 0; a < NA; ++a)
       if (a || b) v[b * NA + a] = cmul(v[b * NA + a], a && b ? cmul(A[a], B) : a ? A[a] : B);
@@ -124,7 +136,7 @@ __device__ __forceinline__ void cfft_twiddle(float2 (&v)[R], int k) {
 // A middle or last pass: R points a butterfly from shared memory; the middle
 // one back to it, the last one to `store`.
 template <int n, int R, int NS, bool COLS, typename Store>
-__device__ __forceinline__ void cfft_pass(float2* buf, int t, int c, Store store) {
+__device__ __forceinline__ void cfft_pass(float2* buf, const float2* table, int t, int c, Store store) {
   constexpr int T = Radices<n>::T, PER = n / R / T;
   constexpr bool last = NS * R == n;
   float2 v[PER][R];
@@ -136,7 +148,7 @@ __device__ __forceinline__ void cfft_pass(float2* buf, int t, int c, Store store
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     const int j = t + u * T, k = j & (NS - 1);
-    cfft_twiddle<R, NS>(v[u], k);
+    cfft_twiddle<R, NS, NS == Radices<n>::R0>(v[u], k, table);
     dft_reg<R>(v[u], TurnW32Exact());
 #pragma unroll
     for (int r = 0; r < R; ++r) {
@@ -201,6 +213,10 @@ k_cfft_inv(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out
       const int i = t + u * T + r * (n / P::R0);
       v[u][r] = mine && i < in_len ? swp(in[q * in_q + i * in_i]) : make_float2(0.f, 0.f);
     }
+  float2* table = cfft_buf + Batch<n, COLS>::POINTS;
+  if constexpr (P::R1 > 1)  // while the points arrive
+    for (int e = threadIdx.x; e < Batch<n, COLS>::TWIDDLES; e += T * C)
+      table[e] = root<P::R0 * P::R1>((e / P::R0 + 1) * (e % P::R0));
 #pragma unroll
   for (int u = 0; u < PER; ++u) {
     dft_reg<P::R0>(v[u], TurnW32Exact());
@@ -212,8 +228,8 @@ k_cfft_inv(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out
   }
   if constexpr (P::R1 > 1) {
     __syncthreads();
-    cfft_pass<n, P::R1, P::R0, COLS>(cfft_buf, t, c, store);
-    if constexpr (P::R2 > 1) cfft_pass<n, P::R2, P::R0 * P::R1, COLS>(cfft_buf, t, c, store);
+    cfft_pass<n, P::R1, P::R0, COLS>(cfft_buf, table, t, c, store);
+    if constexpr (P::R2 > 1) cfft_pass<n, P::R2, P::R0 * P::R1, COLS>(cfft_buf, table, t, c, store);
   }
   if constexpr (PEAK) {
     __threadfence();  // the map's values, for the CTA that reads the peak's
@@ -241,8 +257,7 @@ template <int n, bool COLS, bool PEAK>
 cudaError_t launch_cfft_n(const float2* in, int in_len, int64_t in_q, int64_t in_i, float2* out, int64_t out_q,
                           int64_t out_i, int count, PeakSlot* slot, cudaStream_t st) {
   constexpr int C = Batch<n, COLS>::C;
-  constexpr size_t smem = Radices<n>::R1 == 1 ? 0
-                          : sizeof(float2) * (COLS ? (size_t)n * C : (size_t)C * (n + n / Radices<n>::R0 + 1));
+  constexpr size_t smem = sizeof(float2) * (Batch<n, COLS>::POINTS + Batch<n, COLS>::TWIDDLES);
   cudaError_t e = cudaFuncSetAttribute(k_cfft_inv<n, COLS, PEAK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   k_cfft_inv<n, COLS, PEAK><<<(count + C - 1) / C, Radices<n>::T * C, smem, st>>>(in, in_len, in_q, in_i, out, out_q,
