@@ -197,9 +197,15 @@ __device__ __forceinline__ int cross_source(int S, int a, int b, int pq, bool& f
 }
 
 // A CTA takes one baseline (blockIdx.y) and a run of (subband, hand, channel)
-// values.
-template <bool TC>
+// values, shared by KG groups of threads as in k_finalize: the X step of few
+// rows leaves over a hundred partials (two stations, 1024 channels: 114), whose
+// sum in one chain would round more often than the sums that it adds, and, with
+// few values, is all latency (two stations, 256 channels, 228 partials: 195 us, 12
+// us now).
+template <bool TC, int KG>
 __global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unscale) {
+  constexpr int EL = 256 / KG;
+  __shared__ float2 s_sum[KG > 1 ? 256 : 1];
   const int S = p.S, nsub = p.G, nch = p.nchan;
   const int nblv = nbl_of(2 * S);
   const int bl = blockIdx.y;
@@ -208,32 +214,51 @@ __global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unsca
   while (q >= S - a) { q -= S - a; ++a; }
   const int b = a + q;
   const int per = nsub * 4 * nch;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < per; e += gridDim.x * blockDim.x) {
+  const int g = threadIdx.x / EL;
+  for (int e0 = blockIdx.x * EL; e0 < per; e0 += gridDim.x * EL) {
+    const int e = e0 + threadIdx.x % EL;
+    const bool mine = e < per;
     const int k = e & (nch - 1);  // a power of two of channels
     const int r = e / nch;
     const int pq = r & 3, sb = r >> 2;
     bool flip;
     const int blv = cross_source(S, a, b, pq, flip);
     float2 v = make_float2(0.f, 0.f);
-#pragma unroll 4
-    for (int kz = 0; kz < p.KZ; ++kz) {
+#pragma unroll(KG > 1 ? 8 : 4)
+    for (int kz = g; kz < p.KZ && mine; kz += KG) {
       const float2 x = TC ? p.part[(((size_t)kz * nsub + sb) * nch + k) * nblv + blv]
                           : p.part[(((size_t)kz * nblv + blv) * nsub + sb) * nch + k];
       v.x += x.x;
       v.y += x.y;
     }
+    if constexpr (KG > 1) {
+      __syncthreads();  // the sums of the values before have been read
+      s_sum[threadIdx.x] = v;
+      __syncthreads();
+      if (g != 0) continue;
+      float2 x[KG];  // added up in pairs, with fewer roundings than one by one
+#pragma unroll
+      for (int h = 0; h < KG; ++h) x[h] = s_sum[h * EL + threadIdx.x];
+#pragma unroll
+      for (int h = KG / 2; h > 0; h /= 2)
+#pragma unroll
+        for (int u = 0; u < h; ++u) x[u] = make_float2(x[u].x + x[u + h].x, x[u].y + x[u + h].y);
+      v = x[0];
+    }
     if (flip) v.y = -v.y;
-    p.out[(size_t)bl * per + e] = make_float2(v.x * sc, v.y * sc);
+    if (mine) p.out[(size_t)bl * per + e] = make_float2(v.x * sc, v.y * sc);
   }
 }
 
 cudaError_t launch_finalize_cross(const FinParams& p, bool tc, float unscale, cudaStream_t s) {
-  const int per = p.G * 4 * p.nchan;
-  const dim3 grid(row_ctas(per, 1024, nbl_of(p.S)), nbl_of(p.S));
+  const int per = p.G * 4 * p.nchan, nbl = nbl_of(p.S);
+  const dim3 few(row_ctas(per, 16, nbl), nbl), grid(row_ctas(per, 1024, nbl), nbl);
   if (tc)
-    k_finalize_cross<true><<<grid, 256, 0, s>>>(p, unscale);
+    k_finalize_cross<true, 1><<<grid, 256, 0, s>>>(p, unscale);
+  else if (p.KZ > 8)
+    k_finalize_cross<false, 16><<<few, 256, 0, s>>>(p, unscale);
   else
-    k_finalize_cross<false><<<grid, 256, 0, s>>>(p, unscale);
+    k_finalize_cross<false, 1><<<grid, 256, 0, s>>>(p, unscale);
   return cudaGetLastError();
 }
 
