@@ -15,8 +15,8 @@ namespace corr {
 // Blocks valid at both stations of baseline bl, counted by `threads` threads
 // from index i0; the caller adds their counts up.  Bound by the latency of its
 // loads, which take 16 blocks each where the rows of `valid` start at multiples
-// of 16 bytes (a handle pads them; the static scratch has no room to): 62500
-// blocks took a CTA 120 us with byte loads, 11 us now.
+// of 16 bytes (a handle pads them; in the static scratch they are as long as the
+// integration): 62500 blocks took a CTA 120 us with byte loads, 11 us now.
 __device__ __forceinline__ int count_valid(const FinParams& p, int bl, int i0, int threads) {
   int a = 0, q = bl;  // baseline index -> (a, b)
   while (q >= p.S - a) { q -= p.S - a; ++a; }
@@ -118,18 +118,24 @@ __global__ void __launch_bounds__(256) k_finalize(FinParams p) {
 }
 
 // CTAs along a baseline's elements: one per `each` of them, but no more than
-// fill the SMs a few times over all baselines, since every CTA counts the
-// baseline's valid blocks.
-static unsigned row_ctas(size_t elements, size_t each, int rows) {
-  const size_t need = (elements + each - 1) / each, room = std::max(1, 152 * 32 / rows);
+// `most` an SM over all baselines, since every CTA counts the baseline's valid
+// blocks.
+static unsigned row_ctas(size_t elements, size_t each, int rows, int most = 32) {
+  const size_t need = (elements + each - 1) / each, room = std::max(1, 152 * most / rows);
   return (unsigned)std::min(need, room);
 }
+
+// Sixteen groups of threads share an element's partials where one chain would
+// be long or leave the chip idle: above 8 partials, but for up to 16 of outputs
+// that give every SM a CTA of chains (190 baselines x 12 streams x 256 channels,
+// 9 partials: 55 us in groups, 18 in chains).
+static bool shared_sums(int KZ, size_t values) { return KZ > 16 || (KZ > 8 && values < (size_t)152 * 2048); }
 
 cudaError_t launch_finalize(const FinParams& p, cudaStream_t s) {
   const size_t per = (size_t)p.G * p.nchan;
   const int nbl = nbl_of(p.S);
-  if (p.KZ > 8)
-    k_finalize<16><<<dim3(row_ctas(per, 16, nbl), nbl), 256, 0, s>>>(p);
+  if (shared_sums(p.KZ, per * nbl))
+    k_finalize<16><<<dim3(row_ctas(per, 16, nbl, 8), nbl), 256, 0, s>>>(p);
   else
     k_finalize<1><<<dim3(std::max(row_ctas(per, 2048, nbl), (unsigned)((per + 8191) / 8192)), nbl), 256, 0, s>>>(p);
   return cudaGetLastError();
@@ -252,10 +258,10 @@ __global__ void __launch_bounds__(256) k_finalize_cross(FinParams p, float unsca
 
 cudaError_t launch_finalize_cross(const FinParams& p, bool tc, float unscale, cudaStream_t s) {
   const int per = p.G * 4 * p.nchan, nbl = nbl_of(p.S);
-  const dim3 few(row_ctas(per, 16, nbl), nbl), grid(row_ctas(per, 1024, nbl), nbl);
+  const dim3 few(row_ctas(per, 16, nbl, 8), nbl), grid(row_ctas(per, 1024, nbl), nbl);
   if (tc)
     k_finalize_cross<true, 1><<<grid, 256, 0, s>>>(p, unscale);
-  else if (p.KZ > 8)
+  else if (shared_sums(p.KZ, (size_t)per * nbl))
     k_finalize_cross<false, 16><<<few, 256, 0, s>>>(p, unscale);
   else
     k_finalize_cross<false, 1><<<grid, 256, 0, s>>>(p, unscale);

@@ -369,7 +369,7 @@ k_xpairs(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XPara
       for (int bi = 0; bi < nb; ++bi, st += TS * row_bytes)
         tile_block<TS, 0, DIAG>(acc, st + wa * sh.tile_bytes, st + wb * sh.tile_bytes, row_bytes);
       ring.release(slot);
-        if (++slot == sh.nst) {
+      if (++slot == sh.nst) {
         slot = 0;
         phase ^= 1;
       }
@@ -579,16 +579,22 @@ cudaError_t launch_pairs(const XParams& p_in, const XPlan& x, const XGroups& gro
 
 }  // namespace
 
-// Block ranges per chunk.  At least one per 256 blocks (the length of an FP32
-// register sum); above that the number whose CTAs fill whole waves of the
-// SMs, weighed against each CTA's start and end (worth about 12 blocks) and
-// the partial sums it adds to memory (read and written, against the spectra
-// read).
+// Block ranges per chunk.  At least one per 256 blocks, and where that leaves
+// sums of more than 24 blocks, (but for an eighth) as many as make 912 ranges of
+// 128 channels and 8 x 8 stations: the error of an integration grows with the
+// length of its FP32 register sums (43 stations x 5 streams x 512 channels, 104
+// blocks: 2.65e-7 from 64 bits in three ranges, 2.90e-7 in one).  Above that the
+// number whose CTAs fill whole waves of the SMs, weighed against each CTA's
+// start and end (worth about 12 blocks) and the partial sums it adds to memory
+// (read and written, against the spectra read).
 int xstage_kz(int CB, int S, int G, int nchan) {
   const XPlan x = plan_for(S, nchan, nullptr);
   const int64_t base = (int64_t)x.ngroup * ((nchan + 32 * x.cg - 1) / (32 * x.cg)) * G;
   const int64_t slots = (int64_t)152 * x.ctas_per_sm;
-  const int least = std::max(1, (CB + 255) / 256);
+  const int64_t nt = S <= kOneTile ? 1 : (S + 7) / 8;
+  const int64_t tiles = (int64_t)((nchan + 127) / 128) * G * (nt * (nt + 1) / 2);
+  const int64_t ranges = (912 + tiles - 1) / tiles;
+  const int least = (int)std::max<int64_t>({1, (CB + 255) / 256, std::min<int64_t>((CB + 23) / 24, ranges - ranges / 8)});
   const int most = (int)std::min<int64_t>(CB, std::max<int64_t>(least, 3 * slots / base + 1));
   int best = least;
   double score = 0.0;
