@@ -131,7 +131,8 @@ struct Ring {
   // up, here or in another warp before)
   __device__ __forceinline__ int reclaim(int slot, uint32_t phase) const {
     const int old = slot >= 2 ? slot - 2 : slot - 2 + stages;
-    if (!*abort_flag && ring_wait(&empty[old], old > slot ? phase ^ 1 : phase, abort_flag, limit) && !*abort_flag) return old;
+    const int stop = *abort_flag;  // read first: its latency passes behind the wait's
+    if (ring_wait(&empty[old], old > slot ? phase ^ 1 : phase, abort_flag, limit) && !stop) return old;
     *abort_flag = 1;
     return -1;
   }
