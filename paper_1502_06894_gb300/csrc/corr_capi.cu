@@ -657,6 +657,31 @@ static FParams fparams(corr_t* h, int blk0, int cb, int slot) {
   return p;
 }
 
+namespace corr {
+
+// Blocks per chunk of an integration of M blocks in chunks of at most CB: equal
+// ones in multiples of `unit`, as few as the buffers allow, since a short last
+// one would leave most SMs idle (64 blocks after 19 chunks of 819 cost the time
+// of 120).  Where `group` blocks take `ctas` large CTAs, `slots` at a time (0:
+// where they are small), chunks of CB and a short last one stay unless equal ones
+// take fewer waves: 8192 channels, 4 stations x 16 streams, 256 blocks at most,
+// 2862 blocks: 79 waves, 84 in equal chunks (4.3% of the whole call); operand
+// tiles of 20 stations x 26 streams x 1024 channels, 564 blocks as 512 + 52: 2.27
+// ms, as 320 + 244 2.59 (six waves either way, but the short chunk's one passes
+// during the first chunk's X step).
+int chunk_step(int M, int CB, int unit, int group, int ctas, int slots) {
+  const int n = (M + CB - 1) / CB;
+  const int equal = std::min(CB, ((M + n - 1) / n + unit - 1) / unit * unit);
+  if (ctas <= 0) return equal;
+  auto waves = [&](int step) {
+    auto of = [&](int64_t blocks) { return ((blocks + group - 1) / group * ctas + slots - 1) / slots; };
+    return M / step * of(step) + of(M % step);
+  };
+  return waves(equal) < waves(CB) ? equal : CB;
+}
+
+}  // namespace corr
+
 // Device work of one integration after its delay blocks are in descriptor
 // slot `slot`: F and X per chunk, weights and
 // normalisation, with no host wait (so it can be recorded into a CUDA graph).
@@ -675,14 +700,14 @@ static int enqueue_rest(corr_t* h, cudaStream_t st, int M, float2* vis_out, doub
   // the X step's stations and streams (2S and nsub with both hands)
   const int XS = x_stations(h), XG = x_streams(h);
   cudaStream_t xs = overlap ? h->xstream : st;
-  // chunks of equal length (in whole K tiles on the tensor cores), as few as
-  // the buffers allow: a short last one would leave most SMs idle (64 blocks
-  // after 19 chunks of 819 cost the time of 120)
+  // chunks in whole K tiles on the tensor cores.  Two F kernels run few and
+  // large CTAs: above 4096 channels a block of a station fills an SM (which
+  // counts up to 12 rows, where the F step takes most of the time), and the one
+  // that writes operand tiles takes 8 blocks, two CTAs an SM.
   int step = h->CB;
-  if (h->chunk_req <= 0) {
-    const int n = (M + h->CB - 1) / h->CB, kb = tc ? (fp8 ? 128 : 64) : 1;
-    step = std::min(h->CB, ((M + n - 1) / n + kb - 1) / kb * kb);
-  }
+  if (h->chunk_req <= 0)
+    step = h->tc_direct ? chunk_step(M, h->CB, fp8 ? 128 : 64, 8, S, 2 * h->sm_count)
+                        : chunk_step(M, h->CB, tc ? (fp8 ? 128 : 64) : 1, 1, h->nchan > 4096 && XS <= 12 ? S : 0, h->sm_count);
   int c = 0;
   for (int c0 = 0; c0 < M; c0 += step, ++c) {
     const int buf = overlap ? (c & 1) : 0;
