@@ -1241,6 +1241,8 @@ static cudaError_t launch_LG(const FParams& p, cudaStream_t st) {
     const int rounds = std::max(1, slots * p.G / NGRP);
     const int64_t steps = (int64_t)((p.CB + slots - 1) / slots) * p.S;
     const int64_t most = std::max<int64_t>(1, steps / ((int64_t)4 * ctas * sm_count));
+    // the 8192-point form has one round per stream and stages the next windows into a buffer of their own
+    if (L > 4096 && rounds >= 4) return (int)std::max<int64_t>(1, std::min<int64_t>(4, most / 2));
     return (int)std::min<int64_t>(rounds >= 4 ? 1 : (8 + rounds - 1) / rounds, most);
   };
   // blocks a CTA takes at a time: as many as give every group a transform
