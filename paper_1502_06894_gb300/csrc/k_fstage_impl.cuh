@@ -626,11 +626,13 @@ __device__ __forceinline__ void stage_windows(const FParams& p, const StationVie
     const int64_t a0 = w0 - lead;
     const int ntot = nw + lead;
     const int nvec = ntot >> 2;
-    if (!ASYNC && sv.host) {
+    if (sv.host && (!ASYNC || nvec >= 32)) {
       // pinned host memory over the host link: plain 16-byte loads keep more
-      // of the link's requests in flight than the async copies, which matters
-      // while the CTA waits for its windows (with ASYNC they pass behind a
-      // whole step of transforms)
+      // of the link's requests in flight than the async copies (with ASYNC:
+      // 4 stations x 20 streams x 1024 channels, 6e8 station-samples, 3.59 ms
+      // by copies behind the step before, 2.98 by loads).  Windows of less than
+      // a load for each lane are all latency, which the copies leave behind
+      // that step (one stream x 64 channels: 9.7 ms by loads, 8.5 by copies).
       const uint4* src4 = reinterpret_cast<const uint4*>(sv.words + a0);
       for (int q = tid; q < nvec; q += nt) {
         if (a0 + 4 * q + 4 <= sv.nwords) {
