@@ -383,7 +383,7 @@ static int work_layout(corr_t* h, WorkLayout& w) {
   // no zero padding except in the last chunk of an integration
   if (tc && h->chunk_req <= 0 && cb > kb) cb -= cb % kb;
   w.CB = (int)cb;
-  w.Mcap = (w.Mcap + 15) & ~15;  // rows of block descriptors start at multiples of 16 (k_weights)
+  w.Mcap = (w.Mcap + 15) & ~15;  // rows of block descriptors start at multiples of 16 (count_valid reads 16 at a time)
   w.KZ = xstage_kz(w.CB, XS, XG, nch);
   // tensor-core operand tiles hold up to 64 stations; for FFTs of up to 2048
   // points the F step writes them directly, above that FP16 (FP8) spectra are

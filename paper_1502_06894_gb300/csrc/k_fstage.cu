@@ -4,7 +4,8 @@
 // One CTA takes one station and a few FFT blocks.  Per block it stages the
 // packed 2-bit words of the delay-tracked window [b*N + n_b, +N) in shared
 // memory once (all G streams of a station share one window), turns their codes
-// into words per stream (transforms of 64 to 4096 points), then each FFT group
+// into words per stream (transforms of 64 to 4096 points; post-F ones of 2048
+// points up to 17 streams, beyond which it would cost a CTA per SM), then each FFT group
 // of T threads transforms one stream (k_fstage_impl.cuh; this file holds the
 // dispatch and the tensor-core variant):
 //

@@ -272,9 +272,9 @@ template <> struct Plan<8192> { static constexpr int R0 = 32, R1 = 16, R2 = 16, 
 template <int L> struct Groups {
   static constexpr int T = Plan<L>::T;
   // 256 threads per CTA (64 one-thread transforms for the smallest sizes);
-  // 4096-point complex transforms (8192-sample blocks) run four independent
-  // 256-thread transforms per CTA of 1024 threads, so that barriers stay
-  // within a transform, four of them are in flight per SM and 32 warps hide
+  // 4096-point complex transforms (8192-sample blocks) run three independent
+  // 256-thread transforms per CTA of 768 threads, so that barriers stay
+  // within a transform, three of them are in flight per SM and 24 warps hide
   // the latency of the twiddle loads
   static constexpr int NGRP = T == 1 ? 64 : (L == 4096 ? 3 : 256 / T);
 };
@@ -856,7 +856,7 @@ __device__ __forceinline__ void turn_codes(const uint32_t* __restrict__ wbuf, in
 // CTAs per SM the register allocation must allow: larger FFTs run one group
 // of 128-256 threads per FFT, so without a bound the compiler takes up to
 // 255 registers and a single CTA fills the SM's register file.  (4096- and
-// 8192-point transforms keep one CTA of 512 / 256 threads per SM: their
+// 8192-point transforms keep one CTA of 768 / 256 threads per SM: their
 // buffers and staged windows fill shared memory anyway.)
 template <int L> struct MinBlocks {
   static constexpr int v = (L >= 64 && L <= 1024) ? 2 : (L == 2048 ? 3 : 1);
@@ -909,8 +909,8 @@ __device__ __forceinline__ float2 prerot(int m, float phi0, float dhi, float dlo
 // a (slot, subband), so the CTA forms it once per step (with the accurate sine
 // and cosine) and a point costs one complex product instead of a sine, a
 // cosine and two reductions of its own phase, whose special-function and
-// issue slots bound the pre-F form with the transform's (2048 points: 720 us
-// per 2.7e8 samples, 680 now).
+// issue slots bound the pre-F form with the transform's (2048 points: 705 us
+// per 2.7e8 samples, 680 with the table; 647 now, with the middle pass in place).
 template <int L>
 __device__ __forceinline__ void fill_rotations(const FParams& p, int s, int bb0, int nslots, const int* s_ok, float2* rot) {
   constexpr int R0 = Plan<L>::R0, T = Plan<L>::T;
@@ -960,8 +960,8 @@ __device__ __forceinline__ void rotate_store_pre(V v, int t, float delta, void* 
 // slope.  TURN: the codes come stream by stream from turn_codes, jb streams at
 // a time; else each transform decodes the staged window itself.
 //
-// Bound by the mix of the FMA pipe (48%), the shared-memory pipe (54%) and
-// instruction issue (52%) at the 16 warps that 32 points a thread leave an SM:
+// Bound by the mix of the FMA pipe (51%), the shared-memory pipe (59%) and
+// instruction issue (54%) at the 16 warps that 32 points a thread leave an SM:
 // no one of its parts, taken out, gives more than 9%.  Ten stations x 16
 // streams x 1024 channels, 819 blocks (2.7e8 samples): 328 us; 376 us when each
 // transform decoded the interleaved window (shared-memory pipe 71%) and passed
@@ -1265,7 +1265,7 @@ static cudaError_t launch_LG(const FParams& p, cudaStream_t st) {
       if (jb <= p.G && resident(turned(base, jb)) >= most)
         return launch_turn<L, GC, PRE, true>(p, base, wslot, jb, steps_per_cta(base, most), turned(base, jb), st);
   }
-  if constexpr (!Codes<L, PRE>::on || (L == 2048 && !PRE)) {  // (2048 points, more than 18 streams)
+  if constexpr (!Codes<L, PRE>::on || (L == 2048 && !PRE && GC != 16)) {  // (2048 points, more than 17 streams)
     const size_t one = kWordsOffset<L>(NGRP) + window(base), two = one + window(base);
     const int nseq = resident(two) == MinBlocks<L>::v ? steps_per_cta(base, resident(two)) : 1;
     const size_t smem = nseq > 1 ? two : one;
