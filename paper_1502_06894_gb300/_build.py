@@ -19,7 +19,7 @@ LIB = os.path.join(HERE, "libcorr.so")
 SOURCES = ["k_fstage_small.cu", "k_fstage_pre.cu", "k_fstage_large.cu", "k_fstage_pre_large.cu", "k_fstage.cu",
            "k_fstage_1024.cu", "k_fringe.cu", "k_xstage.cu", "corr_capi.cu", "k_delay.cu", "k_finalize.cu", "k_xmma.cu",
            "corr_static.cu", "corr_server.cu"]
-HEADERS = ["corr_internal.cuh", "k_fstage_impl.cuh", "ring_log.h"]
+HEADERS = ["corr_internal.cuh", "k_fstage_impl.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 

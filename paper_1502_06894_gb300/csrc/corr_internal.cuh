@@ -196,4 +196,30 @@ __host__ __device__ inline unsigned long long coverage_start(int q) { return q =
 __host__ __device__ inline int nbl_of(int S) { return S * (S + 1) / 2; }
 __host__ __device__ inline int bl_index(int a, int b, int S) { return a * S - a * (a - 1) / 2 + (b - a); }
 
+// Which copies a ring of shared-memory stages has in flight (the X step on CUDA
+// cores); on the host for its test.
+//
+// Per slot, the last stage whose copies were issued into it, plus one (0:
+// none).  Several warps issue, and nothing orders the issues of different
+// slots, so that one count of stages could end too small (a copy in flight not
+// seen) or include a stage that was never issued.  A slot's own issues are
+// ordered: stage q goes into slot q % stages, and only after every warp has
+// read stage q - stages.  That also means that a slot's earlier copies have
+// landed, so that the last one is all there is to wait for.
+template <int N>
+struct RingLog {
+  volatile int last[N];
+
+  __host__ __device__ __forceinline__ void clear() {
+    for (int i = 0; i < N; ++i) last[i] = 0;
+  }
+  __host__ __device__ __forceinline__ void note(int slot, int q) { last[slot] = q + 1; }
+  // wait(slot, parity) for the last copies of every slot of a ring of `stages`
+  template <typename Wait>
+  __host__ __device__ __forceinline__ void for_each(int stages, Wait wait) const {
+    for (int slot = 0; slot < stages; ++slot)
+      if (const int n = last[slot]) wait(slot, (unsigned)(((n - 1) / stages) & 1));
+  }
+};
+
 }  // namespace corr

@@ -177,7 +177,7 @@ __device__ __forceinline__ unsigned long long peak_key(float2 v, uint32_t e) {
 // The rows' results lie in the map's own first in_len rows: a CTA of the
 // second pass reads its columns before it writes them, whole 128-byte lines
 // for transforms of up to 512 points, so the search needs no work space.
-// 256 x 1024 values into 512 x 8192 bins: 12.9 + 21.3 us (radix-2 passes in
+// 256 x 1024 values into 512 x 8192 bins: 14.3 + 21.7 us (radix-2 passes in
 // shared memory, a transposed write of the lags and a pass of its own for the
 // peak took 66.6 + 70.7 + 11.0 us).
 template <int n, bool COLS, bool PEAK>

@@ -15,7 +15,6 @@
 // add per element and launch, so results are deterministic and the FP32 sums
 // stay short (hierarchical accumulation).
 #include "corr_internal.cuh"
-#include "ring_log.h"
 
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -305,7 +304,7 @@ k_xmac(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ XParams
 // several blocks per copy (single blocks reach 3.9 TB/s where the FMAs consume
 // 5.5); 16-byte cp.async copies by the multiplying warps took as much of their
 // time again as the multiplications (2.08 ms for 64 stations x 8 streams x
-// 4096 channels x 128 blocks, 1.58 ms now, 44 TFLOP/s; single 8 x 8 pairs took
+// 4096 channels x 128 blocks, 1.60 ms now, 43 TFLOP/s; single 8 x 8 pairs took
 // 3.25 ms).
 template <int TS>
 __global__ void __launch_bounds__(32 * kGroupWarps, 1)

@@ -1,4 +1,4 @@
-"""The X step's record of copies in flight (csrc/ring_log.h), driven on the host.
+"""The X step's record of copies in flight (RingLog), driven on the host.
 
 Stages refilled by neighbouring warps may be issued in either order, and after
 an abort one of two neighbouring stages may not be issued at all.  Whatever the
@@ -11,7 +11,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CSRC = os.path.join(ROOT, "paper_1502_06894_gb300", "csrc")
 
 PROGRAM = r"""
-#include "ring_log.h"
+#include "corr_internal.cuh"
 #include <cstdio>
 
 // Stages [0, n) in a ring of `stages`, the first ring of them in order, then
@@ -63,10 +63,11 @@ int main() {
 
 
 def test_every_copy_in_flight_is_waited_for(tmp_path):
-    src = tmp_path / "t.cpp"
+    from paper_1502_06894_gb300 import _build
+    src = tmp_path / "t.cu"
     src.write_text(PROGRAM)
     exe = str(tmp_path / "t")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, "-o", exe, str(src)], check=True)
+    subprocess.run([_build.nvcc(), *_build.ARCH, "-std=c++17", "-I", CSRC, "-o", exe, str(src)], check=True)
     out = subprocess.run([exe], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout
     assert int(out.stdout.split()[0]) > 10000
