@@ -271,7 +271,8 @@ int corr_rewind(corr_t *h);
 /* Drop all pushed or attached samples and flush state, and rewind; the delay
  * model, format and stream starts are kept.  Also clears a device timeout
  * (CORR_ETIMEOUT) that a correlate call reported, so the handle can be used
- * again. */
+ * again.  Waits for the handle's work; when that fails on a handle that has
+ * correlated, the handle is reset all the same and CORR_ECUDA returned. */
 int corr_reset(corr_t *h);
 
 /* Text of the last error on h (NULL h: last corr_create failure). */
